@@ -136,7 +136,10 @@ long long lsa_op_dof(const lsa_op* op);
 
 /* Bytes of device workspace needed by lsa_phiv / lsa_arnoldi for (op, m, p,
  * precision) on the current device; 0 if the arguments are invalid.  The
- * workspace must be 256-byte aligned.  Its contents need not be initialised. */
+ * workspace must be 256-byte aligned.  Its contents need not be initialised.
+ * In float64 it ends with a second, fixed-point copy of the basis (8 N m bytes,
+ * up to 64 GiB), which the flat kernel's inner products read; the calls also
+ * take a workspace without that part and then convert the columns at each use. */
 size_t lsa_workspace_bytes(const lsa_op* op, int m, int p, int precision);
 
 /* S1 alone: y = A x.  x, y: dev, N elements of the basis type (double for
@@ -349,7 +352,8 @@ lsa_status lsa_expm_phi(const double* H, int ldh, int m, double h, int p, double
  *  is a static device array of LSA_STATIC_WORKSPACE_BYTES inside the library,
  *  held by every GPU that loads the library until the process exits.
  *  Returns LSA_ERR_WORKSPACE when lsa_workspace_bytes(op, min(m, N), p,
- *  precision) exceeds that size (nothing is launched then).
+ *  precision) without the fixed-point copy of the basis exceeds that size
+ *  (nothing is launched then).
  *  The first call on a device looks up the array's device address
  *  (cudaGetSymbolAddress, with that device current); make that first call
  *  before any stream capture.  All calls share the one array and it keeps the

@@ -20,9 +20,16 @@ cudaError_t launch_matvec_adr3d(const ArnoldiParams&, int, const void*, void*, i
 int blocks_per_sm_advdiff2d(int);
 int blocks_per_sm_grayscott2d(int);
 int blocks_per_sm_adr3d(int);
-int flat_blocks_per_sm_adr3d(int);
-int flat_blocks_per_sm_advdiff2d(int);
-int flat_blocks_per_sm_grayscott2d(int);
+cudaError_t launch_arnoldi_flat_advdiff2d(const ArnoldiParams&, int, int, cudaStream_t);
+cudaError_t launch_arnoldi_flat_grayscott2d(const ArnoldiParams&, int, int, cudaStream_t);
+cudaError_t launch_arnoldi_flat_adr3d(const ArnoldiParams&, int, int, cudaStream_t);
+cudaError_t launch_arnoldi_flat_grayscott2d_t(const ArnoldiParams&, int, cudaStream_t);
+cudaError_t launch_arnoldi_flat_grayscott2d_frechet(const ArnoldiParams&, int, cudaStream_t);
+int flat_blocks_per_sm_adr3d(int, int);
+int flat_blocks_per_sm_advdiff2d(int, int);
+int flat_blocks_per_sm_grayscott2d(int, int);
+int flat_blocks_per_sm_grayscott2d_t();
+int flat_blocks_per_sm_grayscott2d_frechet();
 bool tma_applicable_advdiff2d(const DevOp&, const Tiling&, int, int);
 bool tma_applicable_grayscott2d(const DevOp&, const Tiling&, int, int);
 bool tma_applicable_adr3d(const DevOp&, const Tiling&, int, int);
@@ -158,6 +165,9 @@ int arnoldi_blocks_per_sm(const DevOp& d, int precision) {
   return nb;
 }
 
+static int flat_ctas_per_sm(const ArnoldiParams& P, int precision);
+static bool flat_default(const ArnoldiParams& P, int precision);
+
 // The TMA-staged kernel runs the hybrid variants of the float32-basis form
 // whenever its stage buffers fit in shared memory and the grid meets the TMA
 // alignment rules (LSA_TMA=0 in the environment disables it, LSA_TMA=1 also
@@ -212,14 +222,10 @@ static bool use_cluster(const ArnoldiParams& P, int precision) {
 // device, operator shape, m, variant and precision:
 // LSA_TWO_PHASE=0/1/2 in the environment forces it (2 runs form 1 where the
 // flat kernel does not exist); otherwise the form that
-// lsa_tune_step recorded for the shape; otherwise a default measured on
-// GB300: a two-phase form for 3D grids (the z-halo planes make the repeated
-// projection large): the flat one in float64 (ADR 256^3: 93 against 119 ms),
-// the tile one for the float32 basis (where it is used at all: the streaming
-// kernel runs those grids first); the flat form for 2D grids with at least
-// six 16x16 tiles per SM (Gray-Scott 512^2: 9.33 against 9.60 ms in float64,
-// 3.50 against 4.30 in float32), one-pass below that (the extra barrier
-// costs more than the halo).
+// lsa_tune_step recorded for the shape; otherwise the flat form where
+// flat_default says so, the tile two-phase form on other 3D grids (the z-halo
+// planes make the repeated projection large), one-pass on other 2D grids (the
+// extra barrier costs more than the halo).
 struct StepKey {
   int dev, kind, nx, ny, nz, m, variant, precision;
   bool operator<(const StepKey& o) const {
@@ -242,49 +248,73 @@ static bool step_key(const ArnoldiParams& P, int precision, StepKey* k) {
 }
 
 static bool two_phase_applies(const ArnoldiParams& P, int precision) {
-  return is_hybrid(P.variant) && P.naug == 0 && !use_cluster(P, precision) &&
-         !use_stream(P, precision) && !use_tma(P, precision);
+  return is_hybrid(P.variant) && !use_cluster(P, precision) && !use_stream(P, precision) && !use_tma(P, precision);
 }
 
+// The augmented operator runs forms 0 and 2 (the tile two-phase step has no
+// augmented instantiation) and is not tuned.
 static int two_phase_choice(const ArnoldiParams& P, int precision) {
   if (!two_phase_applies(P, precision)) return 0;
   if (g_step_force >= 0) return g_step_force;
   const char* env = getenv("LSA_TWO_PHASE");
   if (env && env[0] >= '0' && env[0] <= '2') return env[0] - '0';
-  StepKey k;
-  if (!step_key(P, precision, &k)) return 0;
-  {
+  if (P.naug == 0) {
+    StepKey k;
+    if (!step_key(P, precision, &k)) return 0;
     std::lock_guard<std::mutex> lock(g_step_mu);
     auto it = g_step_choice.find(k);
     if (it != g_step_choice.end()) return it->second;
   }
-  if (P.op.nz > 1) return precision == LSA_FP64 ? 2 : 1;
-  return P.tl.ntiles >= 6 * sm_count() ? 2 : 0;
+  if (flat_default(P, precision)) return 2;
+  return P.op.nz > 1 ? 1 : 0;
 }
 
-// The flat two-phase kernel exists for the ADR 3D, advection-diffusion and
-// Gray-Scott operators, and its grid must be resident: as many CTAs per SM as
-// the grid kernel's layout assumes.
-static bool flat_fits(const ArnoldiParams& P, int precision) {
-  const int kind = P.op.kind;
-  if (kind != LSA_OP_ADR3D && kind != LSA_OP_ADVDIFF2D && kind != LSA_OP_GRAYSCOTT2D) return false;
-  static int cache[6][2][16];
+// Resident CTAs per SM of the flat two-phase kernel (its grid's barriers need
+// them resident; two at most, which the workspace's partial sums provide for).
+static int flat_ctas_per_sm(const ArnoldiParams& P, int precision) {
+  static int cache[6][2][2][16];
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 16) dev = 0;
-  int& c = cache[kind][precision][dev];
+  const int aug = P.naug > 0;
+  int& c = cache[P.op.kind][precision][aug][dev];
   if (c == 0) {
-    const int nb = kind == LSA_OP_ADR3D ? flat_blocks_per_sm_adr3d(precision)
-                   : kind == LSA_OP_ADVDIFF2D ? flat_blocks_per_sm_advdiff2d(precision)
-                                              : flat_blocks_per_sm_grayscott2d(precision);
-    c = nb >= arnoldi_blocks_per_sm(P.op, precision) ? 1 : -1;
+    int nb = 0;
+    if (P.op.kind == LSA_OP_ADR3D) nb = flat_blocks_per_sm_adr3d(precision, aug);
+    else if (P.op.kind == LSA_OP_ADVDIFF2D) nb = flat_blocks_per_sm_advdiff2d(precision, aug);
+    else if (P.op.kind == LSA_OP_GRAYSCOTT2D) nb = flat_blocks_per_sm_grayscott2d(precision, aug);
+    else if (!aug && precision == LSA_FP64 && P.op.kind == LSA_OP_GRAYSCOTT2D_T) nb = flat_blocks_per_sm_grayscott2d_t();
+    else if (!aug && precision == LSA_FP64) nb = flat_blocks_per_sm_grayscott2d_frechet();
+    c = nb > 0 ? (nb < 2 ? nb : 2) : -1;
   }
-  return c > 0;
+  return c > 0 ? c : 0;
+}
+
+// Where nothing is recorded or forced, the flat kernel runs
+//  * on 3D grids in float64 (256^3, m = 40: 56 ms a phi product, one-pass 161,
+//    tile two-phase 119; 64^3 2.0 against 4.5 ms one-pass);
+//  * on 2D grids of at least six 16 x 16 tiles per SM (Gray-Scott 512^2, m = 64:
+//    6.2 against 10.0 ms one-pass in float64, 2.7 against 4.5 with the float32
+//    basis; 256^2 level);
+//  * for the gradient's operators (Gray-Scott 256^2 gradient 14.1 against 16.2 ms).
+static bool flat_default(const ArnoldiParams& P, int precision) {
+  if (!is_hybrid(P.variant) || flat_ctas_per_sm(P, precision) == 0) return false;
+  if (P.op.kind > LSA_OP_ADR3D) return true;
+  if (P.op.nz > 1) return precision == LSA_FP64;
+  return P.tl.ntiles >= 6 * sm_count();
+}
+
+// CTAs of the flat kernel: every SM's, or fewer so that a share has at least 128 points.
+static int flat_grid(const ArnoldiParams& P, int precision) {
+  const long long want = (P.op.npts + 127) / 128, most = (long long)sm_count() * flat_ctas_per_sm(P, precision);
+  return (int)(want < most ? want : most);
 }
 
 static int step_form(const ArnoldiParams& P, int precision) {
   const int form = two_phase_choice(P, precision);
-  return (form == 2 && !flat_fits(P, precision)) ? 1 : form;
+  if (form == 2 && flat_ctas_per_sm(P, precision) > 0) return 2;
+  if (P.naug > 0) return 0;
+  return form == 0 ? 0 : 1;
 }
 
 static int arnoldi_kernel_kind(const ArnoldiParams& P, int precision) {
@@ -292,7 +322,7 @@ static int arnoldi_kernel_kind(const ArnoldiParams& P, int precision) {
   if (use_stream(P, precision)) return 2;
   if (use_tma(P, precision)) return 1;
   const int form = step_form(P, precision);
-  return form == 0 ? 0 : 3 + form;
+  return form == 0 ? 0 : (form == 1 ? 4 : 5);
 }
 
 static cudaError_t launch_arnoldi_grid(const ArnoldiParams& P, int precision, int G, cudaStream_t s);
@@ -320,6 +350,14 @@ static cudaError_t launch_arnoldi_grid(const ArnoldiParams& P, int precision, in
     if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_arnoldi_tma_advdiff2d(P, precision, maxG, s);
     if (P.op.kind == LSA_OP_GRAYSCOTT2D) return launch_arnoldi_tma_grayscott2d(P, precision, maxG, s);
     return launch_arnoldi_tma_adr3d(P, precision, maxG, s);
+  }
+  if (P.two_phase == 2) {
+    const int F = flat_grid(P, precision);
+    if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_arnoldi_flat_advdiff2d(P, precision, F, s);
+    if (P.op.kind == LSA_OP_GRAYSCOTT2D) return launch_arnoldi_flat_grayscott2d(P, precision, F, s);
+    if (P.op.kind == LSA_OP_GRAYSCOTT2D_T) return launch_arnoldi_flat_grayscott2d_t(P, F, s);
+    if (P.op.kind == LSA_OP_GRAYSCOTT2D_FRECHET) return launch_arnoldi_flat_grayscott2d_frechet(P, F, s);
+    return launch_arnoldi_flat_adr3d(P, precision, F, s);
   }
   if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_arnoldi_advdiff2d(P, precision, G, s);
   if (P.op.kind == LSA_OP_GRAYSCOTT2D) return launch_arnoldi_grayscott2d(P, precision, G, s);
@@ -377,6 +415,11 @@ static bool make_layout(const DevOp& d, int m, int precision, Layout* L) {
   L->E = take(edges ? (size_t)(m + 3) * (size_t)(d.N / 8) * sizeof(float) : 0);
   if (!edges) L->E = 0;
   L->xaug = take((size_t)(m + 3) * PMAX * sizeof(double));
+  // limbs of the basis columns for the flat float64 kernel, last: a workspace that ends before them runs it
+  // with the conversion in place (the fixed workspace of lsa_phiv_noalloc; bases beyond kLimbBytes).
+  L->base = off;
+  L->F = 0;
+  if (precision == LSA_FP64 && limb_bytes(d, m) <= kLimbBytes) L->F = take(limb_bytes(d, m));
   L->total = off;
   L->G = G;
   return true;
@@ -447,7 +490,7 @@ static lsa_status prepare(const lsa_op* op, int m, int precision, void* work, si
   if (pr->d.kind > LSA_OP_ADR3D && precision != LSA_FP64) return LSA_ERR_ARG;
   if (m < 1 || m > MMAX) return LSA_ERR_ARG;
   if (!make_layout(pr->d, m, precision, &pr->L)) return LSA_ERR_CUDA;
-  if (!work || !aligned256(work) || work_bytes < pr->L.total) return LSA_ERR_WORKSPACE;
+  if (!work || !aligned256(work) || work_bytes < pr->L.base) return LSA_ERR_WORKSPACE;
   pr->w = (char*)work;
   if (precision == LSA_FP32_BASIS) {
     pr->d.g0 = (const float*)(pr->w + pr->L.g0);
@@ -467,11 +510,25 @@ static lsa_status prepare(const lsa_op* op, int m, int precision, void* work, si
   P.W1 = pr->w + pr->L.W1;
   P.H = (double*)(pr->w + pr->L.H);
   P.E = pr->L.E ? (float*)(pr->w + pr->L.E) : nullptr;
+  P.F = pr->L.F && work_bytes >= pr->L.total ? (int2*)(pr->w + pr->L.F) : nullptr;
   P.xaug = (double*)(pr->w + pr->L.xaug);
   P.m = m;
   P.brk_tol = precision == LSA_FP64 ? kBreakdownTolFp64 : kBreakdownTolFp32;
   P.timeout_ns = kTimeoutNs;
   return LSA_OK;
+}
+
+static bool workspace_layout(const lsa_op* op, int m, int p, int precision, Layout* L) {
+  DevOp d;
+  if (precision != LSA_FP64 && precision != LSA_FP32_BASIS) return false;
+  if (!make_devop(op, &d) || m < 1 || m > MMAX || p < 0 || p > PMAX) return false;
+  if (d.kind > LSA_OP_ADR3D && precision != LSA_FP64) return false;
+  return make_layout(d, m, precision, L);
+}
+
+size_t workspace_least_bytes(const lsa_op* op, int m, int p, int precision) {
+  Layout L;
+  return workspace_layout(op, m, p, precision, &L) ? L.base : 0;
 }
 
 }  // namespace lsa
@@ -504,13 +561,8 @@ long long lsa_op_dof(const lsa_op* op) {
 }
 
 size_t lsa_workspace_bytes(const lsa_op* op, int m, int p, int precision) {
-  DevOp d;
-  if (precision != LSA_FP64 && precision != LSA_FP32_BASIS) return 0;
-  if (!make_devop(op, &d) || m < 1 || m > MMAX || p < 0 || p > PMAX) return 0;
-  if (d.kind > LSA_OP_ADR3D && precision != LSA_FP64) return 0;
   Layout L;
-  if (!make_layout(d, m, precision, &L)) return 0;
-  return L.total;
+  return workspace_layout(op, m, p, precision, &L) ? L.total : 0;
 }
 
 lsa_status lsa_matvec(const lsa_op* op, const void* x, void* y, int precision, void* work,
@@ -654,7 +706,7 @@ lsa_status lsa_tune_step(const lsa_op* op, const double* v, int m, int variant, 
     cudaEventDestroy(e0);
     return LSA_ERR_CUDA;
   }
-  const int nforms = flat_fits(P, precision) ? 3 : 2;
+  const int nforms = flat_ctas_per_sm(P, precision) > 0 ? 3 : 2;
   float best[3] = {1e30f, 1e30f, 1e30f};
   lsa_status result = LSA_OK;
   for (int form = 0; form < nforms && result == LSA_OK; ++form) {

@@ -293,142 +293,6 @@ struct Engine {
     }
   }
 
-  // Second pass of the flat two-phase step: this CTA's equal flat share of
-  // the grid points (all species of a point together) in chunks of FCH
-  // points.  Each thread forms w = A x at FQ points with the neighbours of x
-  // read through L2 (x was stored by the first pass, before the grid barrier;
-  // the grid is periodic in every direction, as in the tile passes), stores w
-  // and adds the self terms; then the warps form the inner products with basis
-  // columns (warp <-> columns, lane <-> points, as in dots_plane) from the
-  // chunk's x and w in shared memory (xs, ws: NS*FCH values each).  No halo
-  // copy, no tile chain: every CTA has the same number of points.  w is
-  // bitwise the tile passes' value (the operator's own arithmetic on the
-  // loaded values, staged with a row pitch of 2 and species 5 apart); the
-  // inner products sum the points in other groups, so they agree with the
-  // tile passes to rounding.
-  static constexpr int FQ = 2, FCH = FQ * NT;
-  static constexpr bool kFlatOp =
-      Op::KIND == LSA_OP_ADR3D || Op::KIND == LSA_OP_ADVDIFF2D || Op::KIND == LSA_OP_GRAYSCOTT2D;
-  __device__ int run_pass_flat(const PassT<B>& ps, Tc* xs, Tc* ws) {
-    static_assert(kFlatOp, "the flat pass is written for the ADR 3D, advection-diffusion and Gray-Scott operators");
-    const DevOp& d = P.op;
-    const long long np = d.npts;               // grid points (N = NS * np)
-    long long per = (np + gsize - 1) / gsize;
-    per = (per + 31) & ~31LL;
-    const long long e0 = (long long)grank * per;
-    const long long e1 = min(np, e0 + per);
-    const B* xg = ps.srcB;
-    const int nxy = d.nx * d.ny;
-    const bool dx = ps.dmode & DOT_X, dw = ps.dmode & DOT_W;
-    zero_acc();
-    for (long long base = e0; base < e1; base += FCH) {
-#pragma unroll
-      for (int u = 0; u < FQ; ++u) {
-        const int pl = tid + u * NT;
-        Tc xv[NS], wv[NS];
-#pragma unroll
-        for (int sp = 0; sp < NS; ++sp) { xv[sp] = (Tc)0; wv[sp] = (Tc)0; }
-        if (base + pl < e1) {
-          // grid indices in 32 bits, as in the tile passes (N < 2^31)
-          const int q = (int)base + pl;
-          const int r = q / d.nx, ix = q - r * d.nx;
-          const int iz = r / d.ny, iy = r - iz * d.ny;
-          const int qw = ix == 0 ? q + (d.nx - 1) : q - 1;
-          const int qe = ix == d.nx - 1 ? q - (d.nx - 1) : q + 1;
-          const int qs = iy == 0 ? q + (d.ny - 1) * d.nx : q - d.nx;
-          const int qn = iy == d.ny - 1 ? q - (d.ny - 1) * d.nx : q + d.nx;
-          // per species: [south, west, centre, east, north]; below and above at index 2
-          Tc c5[5 * NS], zm[3], zp[3];
-#pragma unroll
-          for (int sp = 0; sp < NS; ++sp) {
-            const B* xsp = xg + (long long)sp * np;
-            c5[5 * sp + 0] = (Tc)__ldcg(xsp + qs);
-            c5[5 * sp + 1] = (Tc)__ldcg(xsp + qw);
-            c5[5 * sp + 2] = (Tc)__ldcg(xsp + q);
-            c5[5 * sp + 3] = (Tc)__ldcg(xsp + qe);
-            c5[5 * sp + 4] = (Tc)__ldcg(xsp + qn);
-          }
-          zm[0] = zm[1] = zp[0] = zp[1] = (Tc)0;
-          if constexpr (DIM == 3) {
-            zm[2] = (Tc)__ldcg(xg + (iz == 0 ? q + (d.nz - 1) * nxy : q - nxy));
-            zp[2] = (Tc)__ldcg(xg + (iz == d.nz - 1 ? q - (d.nz - 1) * nxy : q + nxy));
-          } else {
-            zm[2] = zp[2] = (Tc)0;
-          }
-          Tc out[NS];
-          Op::template apply<Tc, 2, 5>(d, cf, zm, c5, zp, 2, (long long)q, out);
-#pragma unroll
-          for (int sp = 0; sp < NS; ++sp) {
-            Tc w = out[sp];
-            if constexpr (!F64) w = (Tc)(B)w;
-            const Tc x = c5[5 * sp + 2];
-            ps.wout[(long long)sp * np + q] = (B)w;
-            if (ps.self & SELF_XX) self_add(0, x, x);
-            if (ps.self & SELF_XW) self_add(1, x, w);
-            if (ps.self & SELF_WW) self_add(2, w, w);
-            xv[sp] = x;
-            wv[sp] = w;
-          }
-        }
-#pragma unroll
-        for (int sp = 0; sp < NS; ++sp) {
-          xs[sp * FCH + pl] = xv[sp];
-          ws[sp * FCH + pl] = wv[sp];
-        }
-      }
-      __syncthreads();
-      if (ps.d1 > ps.d0) {
-        // lane l takes points l + 32k of the chunk, k < FCH/32, in groups of
-        // 8, one species after the other
-        constexpr int NPL = FCH / 32;
-        const int nv = (int)min((long long)FCH, e1 - base);   // valid points of the chunk
-#pragma unroll 1
-        for (int sp = 0; sp < NS; ++sp) {
-          const Tc* xsp = xs + sp * FCH;
-          const Tc* wsp = ws + sp * FCH;
-#pragma unroll
-          for (int kk = 0; kk < KMAX; ++kk) {
-            const int c = ps.d0 + warp + NW * kk;
-            if (c >= ps.d1) break;
-            const B* col = Vc(c) + (long long)sp * np + base;
-            Tc v[NPL];
-#pragma unroll
-            for (int k = 0; k < NPL; ++k) {
-              const int pl = lane + 32 * k;
-              v[k] = (Tc)__ldcg(col + (pl < nv ? pl : 0));   // beyond the share: x = w = 0 there
-            }
-#pragma unroll
-            for (int g = 0; g < NPL / 8; ++g) {
-              if constexpr (F64) {
-                double a = ax[kk], b = aw[kk];
-#pragma unroll
-                for (int k = 8 * g; k < 8 * g + 8; ++k) {
-                  const int pl = lane + 32 * k;
-                  if (dx) a = fma((double)v[k], (double)xsp[pl], a);
-                  if (dw) b = fma((double)v[k], (double)wsp[pl], b);
-                }
-                ax[kk] = a;
-                aw[kk] = b;
-              } else {
-                float px = 0.f, pw = 0.f;
-#pragma unroll
-                for (int k = 8 * g; k < 8 * g + 8; ++k) {
-                  const int pl = lane + 32 * k;
-                  px = fmaf((float)v[k], (float)xsp[pl], px);
-                  pw = fmaf((float)v[k], (float)wsp[pl], pw);
-                }
-                if (dx) kahan(axs[kk], axc[kk], px);
-                if (dw) kahan(aws[kk], awc[kk], pw);
-              }
-            }
-          }
-        }
-      }
-      __syncthreads();
-    }
-    return write_partials(ps);
-  }
-
   // Stencil at plane z (interior only) from the ring: w = A x.
   __device__ void stencil_plane(const PassT<B>& ps, int x0, int y0, int z, int w, int hg) {
     const DevOp& d = P.op;
@@ -671,6 +535,12 @@ struct Engine {
         else part[c - ps.d0] = (ps.dmode & DOT_X) ? r : 0.0;
       }
     }
+    return write_self(ps, nd);
+  }
+
+  // The self terms' partial sums, after 2 nd dot slots; returns the number of slots.
+  __device__ int write_self(const PassT<B>& ps, int nd) {
+    double* part = P.partials + (long long)grank * SLOTS;
     {
       double r;                              // lane l: value l >> 3
       if constexpr (F64) {
@@ -1124,11 +994,7 @@ struct Engine {
   // x_j = u_j / nrm_est_{j-1} (u_j the projected vector); the normalised
   // v_j = sigma_j x_j with sigma_j = 1/||x_j|| known after step j.  All the
   // rescalings of Alg. 4 are folded into the scalars a, coef and sigma.
-  // kFlat: the instantiation of k_arnoldi_flat, whose two-phase step runs
-  // run_pass_flat after the flat projection (fbuf: 2*NS*FCH values of shared
-  // memory); the other kernels carry none of its code.
-  template <bool kFlat = false>
-  __device__ void run_hybrid(Tc* fbuf = nullptr) {
+  __device__ void run_hybrid() {
     B* V = reinterpret_cast<B*>(P.V);
     B* Wb[2] = {reinterpret_cast<B*>(P.W0), reinterpret_cast<B*>(P.W1)};
     const long long N = P.op.N;
@@ -1162,9 +1028,7 @@ struct Engine {
         ps.srcB = ps.xout;
         ps.xout = nullptr;
       }
-      int ns;
-      if constexpr (kFlat) ns = two ? run_pass_flat(ps, fbuf, fbuf + NS * FCH) : run_pass(ps);
-      else ns = run_pass(ps);
+      const int ns = run_pass(ps);
       if (!reduce_step(gen, ns, j, [&] { hybrid_step(j); }, j - 1)) return;
       if (S.done) return;
       if (S.fallback_pending) {
@@ -1408,25 +1272,6 @@ __global__ void __launch_bounds__(NT, (sizeof(Tc) == 8) ? LSA_MINB_F64 : LSA_MIN
   else e.run_hybrid();
 }
 
-// The hybrid variants with the flat two-phase step (the ADR 3D,
-// advection-diffusion and Gray-Scott operators): a separate instantiation
-// with 2*NS*FCH values of extra shared memory.
-template <class Op, class Tc>
-__global__ void __launch_bounds__(NT, (sizeof(Tc) == 8) ? LSA_MINB_F64 : LSA_MINB_F32)
-    k_arnoldi_flat(ArnoldiParams P) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using E = Engine<Op, Tc, Tc>;
-  typename E::Smem& S = *reinterpret_cast<typename E::Smem*>(smem_raw);
-  E e(P, S, reinterpret_cast<double*>(smem_raw + E::small_offset()));
-  if (!e.place()) return;
-  e.template run_hybrid<true>(reinterpret_cast<Tc*>(smem_raw + E::smem_bytes()));
-}
-
-template <class Op, class Tc>
-size_t flat_smem_bytes() {
-  return Engine<Op, Tc, Tc>::smem_bytes() + 2 * Op::NS * Engine<Op, Tc, Tc>::FCH * sizeof(Tc);
-}
-
 // One stencil pass y = A x with the same tile code (no barrier).
 template <class Op, class Tc, class B>
 __global__ void __launch_bounds__(NT) k_matvec(ArnoldiParams P, const B* x, B* y) {
@@ -1451,12 +1296,6 @@ cudaError_t launch_arnoldi_t(const ArnoldiParams& P, int G, cudaStream_t s) {
     if (P.naug > 0) k = k_arnoldi<Op, Tc, Tc, true>;
   }
   size_t sm = Engine<Op, Tc, Tc>::smem_bytes();
-  if constexpr (Engine<Op, Tc, Tc>::kFlatOp) {
-    if (P.two_phase == 2 && P.naug == 0 && is_hybrid(P.variant)) {
-      k = k_arnoldi_flat<Op, Tc>;
-      sm = flat_smem_bytes<Op, Tc>();
-    }
-  }
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel((void*)k, dim3(G), dim3(NT), args, sm, s);
@@ -1492,24 +1331,6 @@ cudaError_t launch_matvec_op(const ArnoldiParams& P, int precision, const void* 
                              cudaStream_t s) {
   return precision == LSA_FP64 ? launch_matvec_t<Op, double>(P, x, y, G, s)
                                : launch_matvec_t<Op, float>(P, x, y, G, s);
-}
-
-// Resident CTAs per SM of the flat two-phase kernel (0 where it does not exist).
-template <class Op, class Tc>
-int flat_blocks_per_sm_t() {
-  int nb = 0;
-  if constexpr (Engine<Op, Tc, Tc>::kFlatOp) {
-    auto k = k_arnoldi_flat<Op, Tc>;
-    size_t sm = flat_smem_bytes<Op, Tc>();
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, sm);
-  }
-  return nb;
-}
-
-template <class Op>
-int flat_blocks_per_sm_op(int precision) {
-  return precision == LSA_FP64 ? flat_blocks_per_sm_t<Op, double>() : flat_blocks_per_sm_t<Op, float>();
 }
 
 template <class Op>

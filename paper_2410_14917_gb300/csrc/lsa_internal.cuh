@@ -98,10 +98,11 @@ struct ArnoldiParams {
   int m;
   int variant;
   int write_vlast;         // MGS/CGS2: write v_{m+1} (Arnoldi output only)
-  int two_phase;           // hybrid: project, grid barrier, then stencil and inner products
-                           // (no halo projection; one more barrier per step)
+  int two_phase;           // hybrid: 0 one pass; project, grid barrier, then stencil and inner products over the
+                           // tiles (1) or over flat shares (2): no halo projection; one more barrier per step
   double brk_tol;
   long long timeout_ns;
+  int2* F;                 // flat float64 kernel: fixed-point limbs (low, high) of the basis columns (or null)
   float* E;                // streaming float32 kernel: edge array, (m+3) columns of N/8 (or null)
   // Augmented operator of Eqs. 8-9 (phi-function linear combinations): every
   // vector carries naug = p extra entries; Aaug [x; xi] = [A x + B xi; K xi]
@@ -114,7 +115,8 @@ struct ArnoldiParams {
 
 // Workspace layout (all offsets 256-byte aligned).
 struct Layout {
-  size_t ctl, partials, gsum, T, L, H, V, W0, W1, small, coefs, g0, g1, E, xaug, total;
+  size_t ctl, partials, gsum, T, L, H, V, W0, W1, small, coefs, g0, g1, E, F, xaug;
+  size_t base, total;      // without and with the limbs F
   int G;                   // CTAs of the persistent Arnoldi kernel
 };
 
@@ -137,6 +139,14 @@ __host__ __device__ __forceinline__ long long edge_slot(int tiles_x, int tiles_y
 // Host helpers implemented in lsa_api.cu
 bool make_devop(const lsa_op* op, DevOp* d);
 Tiling make_tiling(const DevOp& d);
+// Limbs of m basis columns for the flat float64 kernel: columns padded to whole pairs of values, and reads run
+// up to a piece of points past the last one.
+inline size_t limb_bytes(const DevOp& d, int m) {
+  return ((size_t)d.ns * ((d.npts + 1) & ~1LL) * m + 1024) * sizeof(int2);
+}
+constexpr size_t kLimbBytes = (size_t)64 << 30;   // larger bases are converted in place
+// Bytes that a call needs at least; lsa_workspace_bytes adds the room for the flat kernel's limbs.  0: bad arguments.
+size_t workspace_least_bytes(const lsa_op* op, int m, int p, int precision);
 
 // Launchers implemented per operator translation unit.
 cudaError_t launch_arnoldi(const ArnoldiParams& P, int precision, int G, cudaStream_t s);

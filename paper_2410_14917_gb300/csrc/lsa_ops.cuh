@@ -84,24 +84,24 @@ struct OpGrayScott2D {
 // to v of a loss on phi_1(hA) v (phi_1(hA)^T = phi_1(hA^T)).
 struct OpGrayScott2DT {
   static constexpr int NS = 2, DIM = 2, KIND = LSA_OP_GRAYSCOTT2D_T, NF = 2;
-  template <class Tc, int RP = PW>
+  template <class Tc, int RP = PW, int SP = PS>
   __device__ __forceinline__ static void apply_f(const Coef<Tc>& c, const Tc* zm, const Tc* z0,
                                                  const Tc* zp, int o, Tc f0, Tc f1, Tc* out) {
     (void)zm; (void)zp;
     const Tc a = f1 * f1, b = (Tc)2 * f0 * f1;
     const Tc* U = z0;
-    const Tc* Vv = z0 + PS;
+    const Tc* Vv = z0 + SP;
     Tc u = U[o], v = Vv[o];
     Tc lu = (U[o - 1] + U[o + 1]) + (U[o - RP] + U[o + RP]) - (Tc)4 * u;
     Tc lv = (Vv[o - 1] + Vv[o + 1]) + (Vv[o - RP] + Vv[o + RP]) - (Tc)4 * v;
     out[0] = c.du * lu - (a + c.F) * u + a * v;
     out[1] = c.dv * lv + (b - c.F - c.k) * v - b * u;
   }
-  template <class Tc>
+  template <class Tc, int RP = PW, int SP = PS>
   __device__ __forceinline__ static void apply(const DevOp& d, const Coef<Tc>& c, const Tc* zm,
                                                const Tc* z0, const Tc* zp, int o, long long gpt,
                                                Tc* out) {
-    apply_f<Tc>(c, zm, z0, zp, o, (Tc)__ldg(d.f0 + gpt), (Tc)__ldg(d.f1 + gpt), out);
+    apply_f<Tc, RP, SP>(c, zm, z0, zp, o, (Tc)__ldg(d.f0 + gpt), (Tc)__ldg(d.f1 + gpt), out);
   }
 };
 
@@ -114,7 +114,7 @@ struct OpGrayScott2DT {
 // of the Frechet derivative of exp, applied to Sect. 2.1's Eq. 7 matrix).
 struct OpGrayScottFrechet2D {
   static constexpr int NS = 4, DIM = 2, KIND = LSA_OP_GRAYSCOTT2D_FRECHET, NF = 2;
-  template <class Tc, int RP = PW>
+  template <class Tc, int RP = PW, int SP = PS>
   __device__ __forceinline__ static void apply_f(const Coef<Tc>& c, const Tc* zm, const Tc* z0,
                                                  const Tc* zp, int o, Tc f0, Tc f1, Tc* out) {
     (void)zm; (void)zp;
@@ -122,7 +122,7 @@ struct OpGrayScottFrechet2D {
     Tc x[4], l[4];
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-      const Tc* P = z0 + s * PS;
+      const Tc* P = z0 + s * SP;
       x[s] = P[o];
       l[s] = (P[o - 1] + P[o + 1]) + (P[o - RP] + P[o + RP]) - (Tc)4 * x[s];
     }
@@ -137,11 +137,11 @@ struct OpGrayScottFrechet2D {
     else if (c.dir == 2) { out[0] -= x[2]; out[1] -= x[3]; }
     else out[1] -= x[3];
   }
-  template <class Tc>
+  template <class Tc, int RP = PW, int SP = PS>
   __device__ __forceinline__ static void apply(const DevOp& d, const Coef<Tc>& c, const Tc* zm,
                                                const Tc* z0, const Tc* zp, int o, long long gpt,
                                                Tc* out) {
-    apply_f<Tc>(c, zm, z0, zp, o, (Tc)__ldg(d.f0 + gpt), (Tc)__ldg(d.f1 + gpt), out);
+    apply_f<Tc, RP, SP>(c, zm, z0, zp, o, (Tc)__ldg(d.f0 + gpt), (Tc)__ldg(d.f1 + gpt), out);
   }
 };
 
