@@ -291,17 +291,16 @@ static int flat_ctas_per_sm(const ArnoldiParams& P, int precision) {
 }
 
 // Where nothing is recorded or forced, the flat kernel runs
-//  * on 3D grids in float64 (256^3, m = 40: 56 ms a phi product, one-pass 161,
-//    tile two-phase 119; 64^3 2.0 against 4.5 ms one-pass);
-//  * on 2D grids of at least six 16 x 16 tiles per SM (Gray-Scott 512^2, m = 64:
-//    6.2 against 10.0 ms one-pass in float64, 2.7 against 4.5 with the float32
-//    basis; 256^2 level);
-//  * for the gradient's operators (Gray-Scott 256^2 gradient 14.1 against 16.2 ms).
+//  * in float64 at every size (a phi product on GB300, flat against one-pass:
+//    Gray-Scott 48^2 0.61 and 0.80 ms, 256^2 1.7 and 2.1, 512^2 5.7 and 9.6;
+//    advection-diffusion 97 x 61 0.41 and 0.46; ADR 16^3 0.36 and 0.82);
+//  * with the float32 basis on 2D grids of at least six 16 x 16 tiles per SM
+//    (Gray-Scott 512^2 2.6 against 4.4 ms; below that, and on 3D grids that the
+//    streaming and TMA-staged kernels do not take, the tile forms).
 static bool flat_default(const ArnoldiParams& P, int precision) {
   if (!is_hybrid(P.variant) || flat_ctas_per_sm(P, precision) == 0) return false;
-  if (P.op.kind > LSA_OP_ADR3D) return true;
-  if (P.op.nz > 1) return precision == LSA_FP64;
-  return P.tl.ntiles >= 6 * sm_count();
+  if (precision == LSA_FP64) return true;
+  return P.op.nz == 1 && P.tl.ntiles >= 6 * sm_count();
 }
 
 // CTAs of the flat kernel: every SM's, or fewer so that a share has at least 128 points.
@@ -414,7 +413,6 @@ static bool make_layout(const DevOp& d, int m, int precision, Layout* L) {
                      (d.kind == LSA_OP_ADVDIFF2D || (d.kind == LSA_OP_ADR3D && d.nz % t.ZS == 0));
   L->E = take(edges ? (size_t)(m + 3) * (size_t)(d.N / 8) * sizeof(float) : 0);
   if (!edges) L->E = 0;
-  L->xaug = take((size_t)(m + 3) * PMAX * sizeof(double));
   // limbs of the basis columns for the flat float64 kernel, last: a workspace that ends before them runs it
   // with the conversion in place (the fixed workspace of lsa_phiv_noalloc; bases beyond kLimbBytes).
   L->base = off;
@@ -511,7 +509,6 @@ static lsa_status prepare(const lsa_op* op, int m, int precision, void* work, si
   P.H = (double*)(pr->w + pr->L.H);
   P.E = pr->L.E ? (float*)(pr->w + pr->L.E) : nullptr;
   P.F = pr->L.F && work_bytes >= pr->L.total ? (int2*)(pr->w + pr->L.F) : nullptr;
-  P.xaug = (double*)(pr->w + pr->L.xaug);
   P.m = m;
   P.brk_tol = precision == LSA_FP64 ? kBreakdownTolFp64 : kBreakdownTolFp32;
   P.timeout_ns = kTimeoutNs;

@@ -111,7 +111,7 @@ static lsa_status batch_layout(const lsa_op* ops, const int* ms, int count, int 
   BL->mail = take((size_t)G * sizeof(BatchMail));
   BL->inst = take((size_t)count * sizeof(BatchInst));
   BL->order = take((size_t)count * sizeof(int));
-  BL->partials = take((size_t)G * SLOTS * sizeof(double));
+  BL->partials = take((size_t)2 * G * SLOTS * sizeof(double));
   BL->T = take((size_t)G * MMAX * MMAX * sizeof(double));
   BL->L = take((size_t)G * MMAX * MMAX * sizeof(double));
   BL->mats = take((size_t)G * kMatsPerWorker * sizeof(double));

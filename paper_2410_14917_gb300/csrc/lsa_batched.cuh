@@ -53,7 +53,7 @@ struct BatchCtl {
 // single CTA (its own index).  Workers that run at the same time never share
 // an index.
 struct BatchScratch {
-  double* partials;     // G x SLOTS
+  double* partials;     // 2 G x SLOTS
   double* T;            // G x MMAX^2
   double* L;            // G x MMAX^2
   double* mats;         // G x 6 SMALL_STRIDE^2
@@ -97,8 +97,8 @@ __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchIn
     P.W1 = reinterpret_cast<unsigned char*>(I.V) + (size_t)I.op.N * (I.m + 2) * bs;
     P.H = I.H;
     P.ctl = I.ctl;
-    P.partials = BP.ws.partials + (size_t)wbase * SLOTS;
-    P.gsum = nullptr;
+    P.partials = BP.ws.partials + (size_t)2 * wbase * SLOTS;
+    P.gsum = P.partials + (size_t)gsize * SLOTS;
     P.naug = 0;
     P.T = BP.ws.T + (size_t)wbase * MMAX * MMAX;
     P.L = BP.ws.L + (size_t)wbase * MMAX * MMAX;
@@ -127,10 +127,15 @@ __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchIn
     E e(P, S, small);
     e.grank = grank;
     e.gsize = gsize;
+    e.redundant_steps();
+    e.one_level = true;
     if (P.variant == LSA_MGS) e.run_mgs(false);
     else if (P.variant == LSA_CGS2) e.run_cgs2(false);
     else if (P.variant == LSA_IOCGS) e.run_iocgs(false);
     else e.run_hybrid();
+    // the lead CTA's results (dimension, status, H) are out before any CTA of the group reads them
+    e.bt1 += (unsigned)gsize;
+    if (gsize > 1 && !e.arrive_wait(&I.ctl->arrive, e.bt1, true)) return false;
   }
   __syncthreads();
   if (ld_volatile_i32(&I.ctl->abort_flag)) return false;

@@ -64,14 +64,13 @@ __device__ __forceinline__ void cl_st(int* local, unsigned rank, int v) {
 }
 
 // Shared-memory layout after the engine's (Smem, then the MMAX x MMAX scratch
-// of the O(j^2) step, which holds T between steps in CTA 0): GSMGS's L
-// [MMAX][MMAX], the tile's basis [m+3][CL_TP] (columns 0..m, then the two
+// of the O(j^2) step, which holds T, and GSMGS's L, between steps in CTA 0):
+// the tile's basis [m+3][CL_TP] (columns 0..m, then the two
 // matvec buffers m+1, m+2) and the CTA's partial sums [SLOTS].
 template <class Op>
 struct ClusterLayout {
   using E = Engine<Op, double, double>;
-  static __host__ __device__ constexpr size_t l_off() { return (E::smem_bytes() + 127) & ~(size_t)127; }
-  static __host__ __device__ constexpr size_t vt_off() { return l_off() + sizeof(double) * MMAX * MMAX; }
+  static __host__ __device__ constexpr size_t vt_off() { return (E::smem_bytes() + 127) & ~(size_t)127; }
   static __host__ __device__ constexpr size_t part_off(int m) {
     return vt_off() + sizeof(double) * (size_t)(m + 3) * CL_TP;
   }
@@ -213,6 +212,11 @@ struct ClusterEngine {
   template <class Fn>
   __device__ void reduce(int nslots, int ncoef, Fn fn) {
     __syncthreads();
+    if (e.trow > 0) {                                // CTA 0: the last step's row of T
+      e.trow_slices();
+      __syncthreads();
+      e.trow_finish();
+    }
     cl_sync();     // every CTA's partials are in its shared memory
     if (e.grank == 0) {
       for (int s = e.tid; s < nslots; s += NT) {
@@ -281,7 +285,6 @@ __global__ void __launch_bounds__(NT, 1) k_arnoldi_cluster(ArnoldiParams P, Smal
   e.grank = (int)cl_rank();
   e.gsize = (int)gridDim.x;   // the grid is the cluster
   e.cached = true;            // CTA 0 runs every step: its state stays in shared memory
-  e.smallL = reinterpret_cast<double*>(smem_cl + LY::l_off());
   ClusterEngine<Op> c(e, reinterpret_cast<double*>(smem_cl + LY::vt_off()),
                       reinterpret_cast<double*>(smem_cl + LY::part_off(P.m)));
   c.run_hybrid();

@@ -43,7 +43,8 @@ __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >
 // AUG: the augmented operator of Eqs. 8-9 (phi-function linear combinations;
 // float64 only).  A separate instantiation, so that the plain kernels carry
 // none of its code.
-template <class Op, class Tc, class B, bool AUG = false>
+// TILE: with the shared memory of the tile passes (the flat kernel has its own).
+template <class Op, class Tc, class B, bool AUG = false, bool TILE = true>
 struct Engine {
   static constexpr int NS = Op::NS;
   static constexpr int DIM = Op::DIM;
@@ -52,43 +53,48 @@ struct Engine {
   static constexpr bool F64 = sizeof(Tc) == 8;
 
   struct Smem {
-    Tc ring[RING * NS * PS];
-    Tc wbuf[NS * TX * TY];
+    Tc ring[TILE ? RING * NS * PS : 1];
+    Tc wbuf[TILE ? NS * TX * TY : 1];
     Tc coefc[MMAX + 2];
     double red[SLOTS];
     double tmp[4][MMAX + 2];
     double bred[NW][3];
-    double sj, scale, true_nrm, ss;
-    double xi[PMAX], xw[PMAX];       // augmented operator: extra entries of the pass's x and w
-    int aug_xcol, aug_wcol;          // ... and the columns they belong to (-1: not stored)
+    double sj, scale;
+    // augmented operator: the extra entries of every column, those of the pass's x and w, and the
+    // columns these belong to (-1: not stored)
+    double xaug[AUG ? (MMAX + 3) * PMAX : 1];
+    double xi[PMAX], xw[PMAX];
+    int aug_xcol, aug_wcol;
     Tc a;
-    int flag, done, fallback_pending, stop;
-    // cached mode (one CTA runs every step): lazy scales, norm estimate and
-    // ||A v_j|| of the last step, kept here instead of re-read from global
+    int flag, ok, done, fallback_pending, stop;
+    // lazy scales, norm estimate and ||A v_j|| of the last step, reductions counted so far
     double sig[MMAX + 2];
     double nrm_est_c, aw_prev_c;
-    int syncs_c;                     // reductions counted so far (cached mode)
+    int syncs_c;
   };
 
   const ArnoldiParams& P;
   Smem& S;
-  double* small;                     // MMAX x MMAX scratch: T (every CTA, CWY/NCWY) or the step's staging
-  // Cached mode: the same CTA runs every step (the single-cluster kernel), so T
-  // (and GSMGS's L, in smallL) stay in shared memory between steps, the lazy
-  // scales and scalars are read from S, and the step also leaves the next
-  // pass's coefficients and flags in S (S.coefc, S.a, S.done,
-  // S.fallback_pending).  Global copies are written as in the grid kernels.
-  bool cached = false;
-  double* smallL = nullptr;
-  // Grid kernels running Engine::run_hybrid with the CWY or NCWY correction:
-  // every CTA keeps T in its `small` scratch, one new row per step read in
-  // load_ctl, so that whichever CTA runs the next step need not stage it.
-  bool tcache = false;
+  // MMAX x TS: T below the diagonal (GSMGS: also L, transposed, above it); then the slices of the step's products
+  // with T, NW x 32 (part); then, in the grid kernels, 2 SLOTS places for the sums of few rows
+  double* small;
+  // Cached mode (`small`, the lazy scales and the step's scalars stay in shared
+  // memory between steps): the grid kernels, where every CTA runs every step on
+  // the same reduced sums -- so that nothing has to be published after it --
+  // and the `lead` one writes the results; and CTA 0 of the single-cluster
+  // kernel.  Otherwise (the TMA-staged and streaming kernels, whose scratch
+  // lies in their stage ring) the CTA that completes a reduction runs the step,
+  // with T staged from global memory, and the others read the control block.
+  bool cached = false, lead = true;
+  int trow = 0;                      // cached mode: row of T that finish_trow has to form (0: none)
+  unsigned bt1 = 0, bt2 = 0;         // arrivals that complete the next waits on the two grid counters
+  bool one_level = false;            // batched kernel: order of the float32 form's sums over the CTAs
+  int par = 0;                       // buffer of the partial sums (small grids alternate between two)
   Coef<Tc> cf;
   const int tid, lane, warp;
   int grank, gsize;                  // this CTA's rank in its group and the group size
   __host__ __device__ static constexpr size_t small_offset() { return (sizeof(Smem) + 127) & ~(size_t)127; }
-  __host__ __device__ static constexpr size_t smem_bytes() { return small_offset() + sizeof(double) * MMAX * MMAX; }
+  __host__ __device__ static constexpr size_t smem_bytes() { return small_offset() + sizeof(double) * (STEP_DOUBLES + 2 * SLOTS); }
   // dot accumulators (per lane)
   double ax[KMAX], aw[KMAX];
   float axs[KMAX], axc[KMAX], aws[KMAX], awc[KMAX];
@@ -407,43 +413,53 @@ struct Engine {
   // -------------------------------------------------------------------------
   // Augmented operator (Eqs. 8-9).  The extra entries of a vector follow the
   // same pass formula as its grid points: x_bot = a*src_bot - sum_c coef_c
-  // V_bot,c, and w_bot = K x_bot.  Every CTA forms them at the start of a pass
-  // (p <= PMAX entries, O(p j) work) and the stencil adds B x_bot; CTA rank 0
-  // adds their share to the inner products; the CTA that completes the pass's
-  // reduction stores them (when all CTAs have read the source entries, so an
-  // in-place pass is safe).
+  // V_bot,c, and w_bot = K x_bot.  Every CTA keeps them for all columns in
+  // shared memory and forms those of a pass at its start (one warp per entry,
+  // p <= PMAX of them); the stencil adds B x_bot, CTA rank 0 adds their share
+  // to the inner products, and aug_commit stores them after the pass.
   __device__ __forceinline__ int col_of(const B* ptr) const {
     return (int)((ptr - reinterpret_cast<const B*>(P.V)) / P.op.N);
   }
   __device__ void aug_begin(const PassT<B>& ps) {
+    static_assert(PMAX <= NW, "one warp per extra entry");
     const int p = P.naug;
-    if (tid < p) {
-      double x;
-      if (ps.src64) {            // the start vector: exp(aug_t K) e_p, entry p-1-i = t^i / i!
-        const int i = p - 1 - tid;
-        double v = 1.0;
-        for (int r = 1; r <= i; ++r) v *= P.aug_t / (double)r;
-        x = ps.a * v;
-      } else {
-        x = ps.a * __ldcg(P.xaug + (long long)col_of(ps.srcB) * PMAX + tid);
+    if (warp < p) {
+      double acc = 0.0;
+      for (int c = ps.c0 + lane; c < ps.c1; c += 32) acc = fma((double)S.coefc[c], S.xaug[c * PMAX + warp], acc);
+      acc = warp_sum(acc);
+      if (lane == 0) {
+        double x;
+        if (ps.src64) {          // the start vector: exp(aug_t K) e_p, entry p-1-i = t^i / i!
+          const int i = p - 1 - warp;
+          double v = 1.0;
+          for (int r = 1; r <= i; ++r) v *= P.aug_t / (double)r;
+          x = ps.a * v;
+        } else {
+          x = ps.a * S.xaug[col_of(ps.srcB) * PMAX + warp];
+        }
+        x -= acc;
+        S.xi[warp] = x;
+        if (warp > 0) S.xw[warp - 1] = x;
+        if (warp == p - 1) S.xw[warp] = 0.0;
       }
-      for (int c = ps.c0; c < ps.c1; ++c)
-        x = fma(-(double)S.coefc[c], __ldcg(P.xaug + (long long)c * PMAX + tid), x);
-      S.xi[tid] = x;
     }
     if (tid == 0) {
       S.aug_xcol = ps.xout ? col_of(ps.xout) : -1;
       S.aug_wcol = ps.wout ? col_of(ps.wout) : -1;
     }
     __syncthreads();
-    if (tid < p) S.xw[tid] = (tid + 1 < p) ? S.xi[tid + 1] : 0.0;
-    __syncthreads();
+  }
+  __device__ void aug_commit() {
+    if (tid < P.naug) {
+      if (S.aug_xcol >= 0) S.xaug[S.aug_xcol * PMAX + tid] = S.xi[tid];
+      if (S.aug_wcol >= 0) S.xaug[S.aug_wcol * PMAX + tid] = S.xw[tid];
+    }
   }
   // extra-entry share of (column c) . (x or w)
   __device__ double aug_dot(int c, const double* vec) const {
     double acc = 0.0;
     for (int k = 0; k < P.naug; ++k) {
-      const double vc = (c == S.aug_xcol) ? S.xi[k] : __ldcg(P.xaug + (long long)c * PMAX + k);
+      const double vc = (c == S.aug_xcol) ? S.xi[k] : S.xaug[c * PMAX + k];
       acc = fma(vc, vec[k], acc);
     }
     return acc;
@@ -503,7 +519,7 @@ struct Engine {
   __device__ int write_partials(const PassT<B>& ps) {
     static_assert(KMAX == 8, "the transposed warp sum below takes 2*KMAX = 16 values");
     const int nd = ps.d1 > ps.d0 ? ps.d1 - ps.d0 : 0;
-    double* part = P.partials + (long long)grank * SLOTS;
+    double* part = part_row();
     {
       // the warp's 2*KMAX column sums at once: value 2kk is x . V_c, 2kk+1 is
       // w . V_c for column c = d0 + warp + NW*kk; lanes 2k and 2k+1 get value k
@@ -540,7 +556,7 @@ struct Engine {
 
   // The self terms' partial sums, after 2 nd dot slots; returns the number of slots.
   __device__ int write_self(const PassT<B>& ps, int nd) {
-    double* part = P.partials + (long long)grank * SLOTS;
+    double* part = part_row();
     {
       double r;                              // lane l: value l >> 3
       if constexpr (F64) {
@@ -565,34 +581,16 @@ struct Engine {
     return 2 * nd + 3;
   }
 
-  // Last CTA: fixed-order reduction of all CTAs' partials into S.red.  Warp w
-  // takes slots w, w+NW, ...; lane l sums CTAs l, l+32, ... in order (all its
-  // loads are independent, so they are in flight together), then a fixed
-  // butterfly combines the lanes: the result is deterministic for a given grid.
-  __device__ void reduce_partials(int nslots) {
-    const int G = gsize;
-    for (int s = warp; s < nslots; s += NW) {
-      const double* ps = P.partials + s;
-      double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-      int c = lane;
-      for (; c + 96 < G; c += 128) {
-        a0 += __ldcg(ps + (long long)c * SLOTS);
-        a1 += __ldcg(ps + (long long)(c + 32) * SLOTS);
-        a2 += __ldcg(ps + (long long)(c + 64) * SLOTS);
-        a3 += __ldcg(ps + (long long)(c + 96) * SLOTS);
-      }
-      for (; c < G; c += 32) a0 += __ldcg(ps + (long long)c * SLOTS);
-      double v = warp_sum((a0 + a1) + (a2 + a3));
-      if (lane == 0) S.red[s] = v;
-    }
-    __syncthreads();
+  __device__ __forceinline__ double* part(int w) const { return small + MMAX * TS + w * 32; }
+
+  // This CTA's row of partial sums.
+  __device__ __forceinline__ double* part_row() const {
+    return (par ? P.gsum : P.partials) + (long long)grank * SLOTS;
   }
 
-  // Two-level form.  Level 1: the last CTA of group g (CTAs g*RG .. g*RG+gn-1)
-  // sums the group's partials into gsum row g; level 2: the last group to
-  // finish sums the group rows into S.red.  One thread per slot, so the loads
-  // of a warp are contiguous; each thread adds its rows in index order, so the
-  // result is deterministic for a given grid.
+  // dst[s] = sum of nrows rows of partial sums.  One thread per slot, so the
+  // loads of a warp are contiguous; each thread adds its rows in index order,
+  // so the result is deterministic for a given grid.
   __device__ void sum_rows(const double* src, int nrows, int nslots, double* dst, bool to_smem) {
     for (int s = tid; s < nslots; s += NT) {
       double acc = 0.0;
@@ -628,11 +626,7 @@ struct Engine {
       S.tmp[0][0] = (double)sm;
       S.tmp[0][1] = (double)slot;
     }
-    const BarrierRef br{&P.ctl->p_arrive, &P.ctl->p_release, &P.ctl->abort_flag, &P.ctl->status};
-    const int r = barrier_arrive(br, 0u, gsize, &S.flag, P.timeout_ns);
-    if (r < 0) return false;
-    if (r == 1) barrier_release(br, 0u);
-    __syncthreads();
+    if (!arrive_wait(&P.ctl->p_arrive, gsize, true)) return false;
     if (warp == 0) {
       const unsigned sm = (unsigned)S.tmp[0][0], slot = (unsigned)S.tmp[0][1];
       int rank = 0;
@@ -649,17 +643,208 @@ struct Engine {
     return true;
   }
 
+  // Arrival at a grid counter (when `arrive`) and the wait until it has counted
+  // `target`, bounded like barrier_arrive's; false on a timeout or abort.  One
+  // atomic and one polled word, which is about 1.5 us less than an arrival
+  // whose last CTA sets a release flag.  Memory ordering as in barrier_arrive.
+  // The pending row of T is formed between the arrival and the wait.
+  __device__ bool arrive_wait(unsigned* ctr, unsigned target, bool arrive) {
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (arrive) atomicAdd(ctr, 1u);
+    }
+    if (trow > 0) trow_slices();
+    if (tid == 0) {
+      int ok = 1;
+      unsigned it = 0;
+      const unsigned long long t0 = global_ns();
+      while ((int)(ld_acquire_u32(ctr) - target) < 0) {
+        if ((++it & 255u) == 0u) {
+          if (ld_volatile_i32(&P.ctl->abort_flag)) { ok = 0; break; }
+          if ((long long)(global_ns() - t0) > P.timeout_ns) {
+            atomicExch(&P.ctl->abort_flag, 1);
+            atomicCAS(&P.ctl->status, 0, (int)LSA_ERR_TIMEOUT);
+            ok = 0;
+            break;
+          }
+          if (it > 4096u) __nanosleep(64);
+        }
+      }
+      __threadfence();
+      S.ok = ok;
+    }
+    __syncthreads();
+    if (trow > 0) trow_finish();
+    return S.ok != 0;
+  }
+
+  // Reduction of a pass's partial sums by every CTA.  Up to DIRECT CTAs each
+  // sums all the rows after one barrier (two buffers of rows in turn, so that a
+  // fast CTA's next row does not overwrite one that is still read).  Larger
+  // grids: CTA q sums slots 4q..4q+3 of all rows, a second barrier, and every
+  // CTA reads the sums.  Then `fn` runs in every CTA with S.red filled, so
+  // nothing is published after it.  All sums run in a fixed order.
+  static constexpr int DIRECT = 48;
+  template <class Fn>
+  __device__ bool reduce_all(int nslots, Fn fn) {
+    bt1 += (unsigned)gsize;
+    if (!arrive_wait(&P.ctl->arrive, bt1, true)) return false;
+    if (gsize <= DIRECT) {
+      const double* src = par ? P.gsum : P.partials;
+      if constexpr (F64) sum_few(src, gsize, nslots);
+      else sum_few_ordered(src, gsize, nslots);
+      par ^= 1;
+    } else {
+      const int nq = (nslots + 3) / 4;
+      if (grank < nq) {
+        if constexpr (F64) sum_slots(4 * grank);
+        else sum_slots_ordered(4 * grank);
+      }
+      bt2 += (unsigned)nq;
+      if (!arrive_wait(&P.ctl->release, bt2, grank < nq)) return false;
+      for (int s = tid; s < nslots; s += NT) S.red[s] = __ldcg(P.gsum + s);
+    }
+    if (AUG) aug_commit();
+    if (lead && tid == 0) atomicAdd(&P.ctl->barriers, 1);
+    __syncthreads();
+    fn();
+    __syncthreads();
+    return true;
+  }
+
+  // S.red[s] = sum of up to DIRECT rows of partial sums: as many threads per slot as there are (a power of
+  // two), each with a run of the rows in one round trip to L2 where they fit, their sums added in order.
+  __device__ void sum_few(const double* src, int nrows, int nslots) {
+    int ng = 1;
+    while (ng < 8 && 2 * ng * nslots <= NT && ng < nrows) ng *= 2;
+    const int per = (nrows + ng - 1) / ng;
+    double* scratch = small + STEP_DOUBLES;
+    for (int i = tid; i < ng * nslots; i += NT) {
+      const int g = i / nslots, s = i - g * nslots;
+      const int r0 = g * per, r1 = min(nrows, r0 + per);
+      double acc = 0.0;
+      for (int r = r0; r < r1; r += 16) {
+        double v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = (r + k < r1) ? __ldcg(src + (long long)(r + k) * SLOTS + s) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (r + k < r1) acc += v[k];
+      }
+      if (ng == 1) S.red[s] = acc;
+      else scratch[i] = acc;
+    }
+    if (ng > 1) {
+      __syncthreads();
+      for (int s = tid; s < nslots; s += NT) {
+        double acc = scratch[s];
+        for (int g = 1; g < ng; ++g) acc += scratch[g * nslots + s];
+        S.red[s] = acc;
+      }
+    }
+  }
+
+  // gsum[s0..s0+3] = the sums of these slots over all rows: thread t takes rows t, t + NT, ...
+  __device__ void sum_slots(int s0) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int r = tid; r < gsize; r += NT) {
+      const double2* row = reinterpret_cast<const double2*>(P.partials + (long long)r * SLOTS + s0);
+      const double2 a = __ldcg(row), b = __ldcg(row + 1);
+      v[0] += a.x; v[1] += a.y; v[2] += b.x; v[3] += b.y;
+    }
+    const double t = warp_sum_many<4>(v);            // lane l: value l >> 3
+    if ((lane & 7) == 0) S.tmp[3][warp * 4 + (lane >> 3)] = t;
+    __syncthreads();
+    if (tid < 4) {
+      double acc = 0.0;
+      for (int i = 0; i < NW; ++i) acc += S.tmp[3][i * 4 + tid];
+      __stcg(P.gsum + s0 + tid, acc);
+    }
+  }
+
+  // The same sums of the float32 form, in one order whatever the reduction's shape (see hybrid_step_ordered):
+  // rows in index order within groups of RG, then the groups; in the batched kernel (one_level) lane by lane.
+  __device__ double run_sum(const double* src, int r0, int r1) const {
+    double acc = 0.0;
+    for (int r = r0; r < r1; r += 16) {
+      double v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = (r + k < r1) ? __ldcg(src + (long long)(r + k) * SLOTS) : 0.0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (r + k < r1) acc += v[k];
+    }
+    return acc;
+  }
+  __device__ double lane_sum(const double* src) const {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    int c = lane;
+    for (; c + 96 < gsize; c += 128) {
+      a0 += __ldcg(src + (long long)c * SLOTS);
+      a1 += __ldcg(src + (long long)(c + 32) * SLOTS);
+      a2 += __ldcg(src + (long long)(c + 64) * SLOTS);
+      a3 += __ldcg(src + (long long)(c + 96) * SLOTS);
+    }
+    for (; c < gsize; c += 32) a0 += __ldcg(src + (long long)c * SLOTS);
+    return warp_sum((a0 + a1) + (a2 + a3));
+  }
+  __device__ void sum_few_ordered(const double* src, int nrows, int nslots) {
+    if (one_level) {
+      for (int s = warp; s < nslots; s += NW) {
+        const double v = lane_sum(src + s);
+        if (lane == 0) S.red[s] = v;
+      }
+      return;
+    }
+    static_assert(DIRECT <= 2 * RG, "at most two groups");
+    double* scratch = small + STEP_DOUBLES;
+    const int ngr = (nrows + RG - 1) / RG;
+    for (int i = tid; i < ngr * nslots; i += NT) {
+      const int g = i / nslots, s = i - g * nslots;
+      scratch[g * SLOTS + s] = run_sum(src + s, g * RG, min(nrows, (g + 1) * RG));
+    }
+    __syncthreads();
+    for (int s = tid; s < nslots; s += NT) {
+      double acc = 0.0;
+      for (int g = 0; g < ngr; ++g) acc += scratch[g * SLOTS + s];
+      S.red[s] = acc;
+    }
+  }
+  __device__ void sum_slots_ordered(int s0) {
+    if (one_level) {
+      if (warp < 4) {
+        const double v = lane_sum(P.partials + s0 + warp);
+        if (lane == 0) __stcg(P.gsum + s0 + warp, v);
+      }
+      return;
+    }
+    double* scratch = small + STEP_DOUBLES;
+    const int ngr = (gsize + RG - 1) / RG, s = tid & 3, g = tid >> 2;
+    if (g < ngr) scratch[tid] = run_sum(P.partials + s0 + s, g * RG, min(gsize, (g + 1) * RG));
+    __syncthreads();
+    if (tid < 4) {
+      double acc = 0.0;
+      for (int i = 0; i < ngr; ++i) acc += scratch[4 * i + tid];
+      __stcg(P.gsum + s0 + tid, acc);
+    }
+  }
+
+  // Every CTA runs the steps from here on (grid kernels, after place()).
+  __device__ void redundant_steps() {
+    cached = true;
+    lead = grank == 0;
+  }
+
   // Read the published control state into shared memory (all threads): the
   // next pass's coefficients and flags, and the hybrid step's lazy scales,
   // norm estimate, ||A v|| and reduction count, so that whichever CTA runs
   // the next step finds them here (no L2 round trip inside the step).
-  __device__ void load_ctl(int ncoef, int trow = -1) {
+  __device__ void load_ctl(int ncoef) {
     for (int c = tid; c < ncoef; c += NT) {
       S.coefc[c] = (Tc)__ldcg(&P.ctl->coef[c]);
       S.sig[c] = __ldcg(&P.ctl->sigma[c]);
     }
-    if (tcache && trow > 0)
-      for (int k = tid; k < trow; k += NT) small[trow * MMAX + k] = __ldcg(&P.T[trow * MMAX + k]);
     if (tid == 0) {
       S.a = (Tc)__ldcg(&P.ctl->a);
       S.done = __ldcg(&P.ctl->done);
@@ -671,70 +856,56 @@ struct Engine {
     __syncthreads();
   }
 
-  // Barrier + reduction; `fn` runs in the last CTA with S.red filled.
+  // Barrier + two-level reduction whose last CTA runs `fn` (the TMA-staged and
+  // streaming kernels): the last CTA of each group of RG sums the group's rows,
+  // the last group to finish sums the group sums into S.red, runs the step and
+  // releases the others, which read the control block.
   template <class Fn>
-  __device__ bool reduce_step(unsigned& gen, int nslots, int ncoef_after, Fn fn, int trow = -1) {
+  __device__ bool reduce_step(unsigned& gen, int nslots, int ncoef_after, Fn fn) {
     const BarrierRef br = arnoldi_barrier(P.ctl);
-    int r;
-    if (P.gsum == nullptr || gsize > RG * RG_MAX) {
-      r = barrier_arrive(br, gen, gsize, &S.flag, P.timeout_ns);
-      if (r == 1) reduce_partials(nslots);
-    } else {
-      const int grp = grank / RG, g0 = grp * RG;
-      const int gn = min(RG, gsize - g0), ngr = (gsize + RG - 1) / RG;
-      const int lead = counter_arrive(&P.ctl->g_arrive[grp], gen, gn, &S.flag);
-      if (lead) sum_rows(P.partials + (long long)g0 * SLOTS, gn, nslots, P.gsum + (long long)grp * SLOTS, false);
-      r = barrier_arrive(br, gen, ngr, &S.flag, P.timeout_ns, lead != 0);
-      if (r == 1) {
-        sum_rows(P.gsum, ngr, nslots, S.red, true);
-        __syncthreads();
-      }
-    }
+    const int grp = grank / RG, g0 = grp * RG;
+    const int gn = min(RG, gsize - g0), ngr = (gsize + RG - 1) / RG;
+    const int last = counter_arrive(&P.ctl->g_arrive[grp], gen, gn, &S.flag);
+    if (last) sum_rows(P.partials + (long long)g0 * SLOTS, gn, nslots, P.gsum + (long long)grp * SLOTS, false);
+    const int r = barrier_arrive(br, gen, ngr, &S.flag, P.timeout_ns, last != 0);
     if (r < 0) return false;
     if (r == 1) {
-      if (AUG && tid < P.naug) {
-        if (S.aug_xcol >= 0) P.xaug[(long long)S.aug_xcol * PMAX + tid] = S.xi[tid];
-        if (S.aug_wcol >= 0) P.xaug[(long long)S.aug_wcol * PMAX + tid] = S.xw[tid];
-      }
+      sum_rows(P.gsum, ngr, nslots, S.red, true);
+      __syncthreads();
       fn();
       __syncthreads();
       if (tid == 0) atomicAdd(&P.ctl->barriers, 1);
       barrier_release(br, gen);
     }
     ++gen;
-    load_ctl(ncoef_after, trow);
+    load_ctl(ncoef_after);
     return true;
   }
 
-  // Grid barrier without a reduction (between the two passes of the
-  // two-phase step), with the arrival structure of reduce_step.
-  __device__ bool sync_only(unsigned& gen) {
-    const BarrierRef br = arnoldi_barrier(P.ctl);
-    int r;
-    if (P.gsum == nullptr || gsize > RG * RG_MAX) {
-      r = barrier_arrive(br, gen, gsize, &S.flag, P.timeout_ns);
-    } else {
-      const int grp = grank / RG, g0 = grp * RG;
-      const int gn = min(RG, gsize - g0), ngr = (gsize + RG - 1) / RG;
-      const int lead = counter_arrive(&P.ctl->g_arrive[grp], gen, gn, &S.flag);
-      r = barrier_arrive(br, gen, ngr, &S.flag, P.timeout_ns, lead != 0);
-    }
-    if (r < 0) return false;
-    if (r == 1) {
-      if (tid == 0) atomicAdd(&P.ctl->barriers, 1);
-      barrier_release(br, gen);
-    }
-    ++gen;
-    return true;
+  // Grid barrier without a reduction (between the two passes of the two-phase step).
+  __device__ bool sync_only() {
+    bt1 += (unsigned)gsize;
+    if (lead && tid == 0) atomicAdd(&P.ctl->barriers, 1);
+    return arrive_wait(&P.ctl->arrive, bt1, true);
   }
 
   __device__ __forceinline__ double& Hat(int r, int c) const { return P.H[r + (long long)c * (P.m + 1)]; }
 
   // -------------------------------------------------------------------------
-  // Hybrid low-synchronisation step (Alg. 4 with Alg. 5/6/7), last CTA only.
+  // Hybrid low-synchronisation step (Alg. 4 with Alg. 5/6/7).
   // S.red: x_i.x_j (i < j-1), x_i.w_j (i < j-1), x_j.x_j, x_j.w_j, w_j.w_j for the
   // stored (estimate-normalised) x and w = A x.
+  // The critical path of every Arnoldi step: float64 instructions take 16
+  // clocks per warp and long latencies, so it is kept short.  Row j of T is not
+  // on it: the last entry of h = T_j t2 (t1, t2 the scaled sums) is
+  // t2_j - t1 . (T_{j-1} t2), and T's row is formed while the next reduction
+  // waits (finish_trow).  The norm estimate needs t2 only, and one warp forms
+  // it beside the others' product with T.
   __device__ void hybrid_step(int j) {
+    if (!F64 || !cached) {
+      hybrid_step_ordered(j);
+      return;
+    }
     Ctl* ctl = P.ctl;
     const int np = j - 1;
     double* temp1 = S.tmp[0];
@@ -744,16 +915,219 @@ struct Engine {
     if (tid == 0) {
       double Gj = S.red[2 * np], Pj = S.red[2 * np + 1], Q = S.red[2 * np + 2];
       S.flag = 0;
+      const int syncs = ++S.syncs_c;
+      if (lead) ctl->syncs = syncs;
       if (j == 1 && Gj == 0.0) {              // zero start vector: y = 0
-        ctl->beta = 0.0;
-        ctl->m_eff = 0;
-        ctl->done = 1;
         S.flag = 1;
+        if (lead) { ctl->beta = 0.0; ctl->m_eff = 0; ctl->done = 1; }
       } else if (!(Gj > 0.0) || !isfinite(Gj) || !isfinite(Pj) || !isfinite(Q)) {
-        ctl->status = (int)LSA_ERR_NUMERIC;
-        ctl->done = 1;
-        ctl->m_eff = j - 1;
         S.flag = 1;
+        if (lead) { ctl->status = (int)LSA_ERR_NUMERIC; ctl->done = 1; ctl->m_eff = j - 1; }
+      } else {
+        // one reciprocal square root for both 1/||x|| and ||x||
+        const double sj = rsqrt(Gj);
+        const double nx = Gj * sj;
+        S.sj = sj;
+        if (j == 1) {
+          if (lead) ctl->beta = nx;
+        } else {
+          const double tn = S.nrm_est_c * nx;              // true norm of the previous vector
+          if (lead) Hat(j - 1, j - 2) = tn;
+          if (!(tn > P.brk_tol * S.aw_prev_c)) {           // lagged breakdown test
+            S.flag = 1;
+            if (lead) { ctl->m_eff = j - 1; ctl->breakdown = 1; ctl->done = 1; }
+          }
+        }
+        if (lead) ctl->sigma[j - 1] = sj;
+        S.sig[j - 1] = sj;
+        temp2[np] = sj * sj * Pj;
+        temp2[np + 1] = sj * sj * Q;
+      }
+      if (S.flag) S.done = 1;
+    }
+    __syncthreads();
+    if (S.flag) return;
+    for (int i = tid; i < 2 * np; i += NT) {
+      const int k = i < np ? i : i - np;
+      (i < np ? temp1 : temp2)[k] = S.sig[k] * S.sj * S.red[i];
+    }
+    __syncthreads();
+    // T_{j-1} temp2 (Alg. 7: M^{-1} temp2) by warps 1..7, and the norm estimate in warp 0
+    if (warp == 0) norm_estimate(j, temp2);
+    else lower_slices(temp2, np);
+    __syncthreads();
+    double* y = P.variant == LSA_HGSMGS ? aux : hcol;
+    if (warp == 0) {
+      // lane l: rows l and l + 32; then the last entry, t2_j + (row j of T) . t2 = t2_j - t1 . y
+      double acc = 0.0;
+      const double* r = P.variant == LSA_HNCWY ? temp2 : y;
+#pragma unroll
+      for (int i = lane; i < MMAX; i += 32)
+        if (i < np) {
+          y[i] = lower_row(temp2, i);
+          acc = fma(temp1[i], r[i], acc);
+        }
+      const double h = temp2[np] - warp_sum(acc);
+      if (lane == 0) y[np] = h;
+      __syncwarp();
+      if (P.variant != LSA_HGSMGS)
+        for (int i = lane; i < j; i += 32) set_coef(i, j, y[i]);
+    }
+    if (P.variant == LSA_HGSMGS) {
+      __syncthreads();
+      gauss_seidel(j, temp1, temp2, aux, hcol);
+      __syncthreads();
+      for (int i = tid; i < j; i += NT) set_coef(i, j, hcol[i]);
+    }
+    trow = np;
+  }
+
+  // H_{i+1,j} = h and the coefficient of column i in the next projection.
+  __device__ __forceinline__ void set_coef(int i, int j, double h) {
+    const double c = S.sig[i] * h * S.scale;
+    if (lead) Hat(i, j - 1) = h;
+    S.coefc[i] = (Tc)c;
+  }
+
+  // Eq. 18 (warp 0): ||v_{j+1}||^2 ~ t - |temp2_{1:j}|^2 with t = ||A v_j||^2.
+  __device__ void norm_estimate(int j, const double* temp2) {
+    Ctl* ctl = P.ctl;
+    double ss = 0.0;
+    for (int i = lane; i < j; i += 32) ss = fma(temp2[i], temp2[i], ss);
+    ss = warp_sum(ss);
+    const double t = temp2[j];
+    // both reciprocal square roots at once: lane 0 that of t - ss, the others that of t
+    const double v = lane == 0 ? t - ss : t;
+    const double r = (v > 0.0) ? rsqrt(v) : 0.0;
+    const double root = v * r;
+    const double awn = __shfl_sync(0xffffffffu, root, 1);
+    if (lane == 0) {
+      bool done_now = false;
+      double ne = 1.0, scale = 1.0;
+      if (t < ss) {                           // Pythagorean radicand negative: explicit norm
+        if (lead) { atomicAdd(&ctl->fallbacks, 1); ctl->fallback_pending = 1; }
+        S.fallback_pending = 1;
+      } else {
+        ne = root;
+        scale = r;
+        if (!(ne > P.brk_tol * awn)) {
+          if (lead) { Hat(j, j - 1) = ne; ctl->m_eff = j; ctl->breakdown = 1; ctl->done = 1; }
+          S.done = 1;
+          done_now = true;
+        }
+      }
+      S.scale = scale;
+      S.nrm_est_c = ne;
+      S.aw_prev_c = awn;
+      S.a = (Tc)(S.sj * scale);
+      if (lead) {
+        ctl->nrm_est = ne;
+        ctl->aw_prev = awn;
+        ctl->a = S.sj * scale;
+        if (j == P.m && !done_now) ctl->m_eff = P.m;
+      }
+    }
+  }
+
+  // sum_{k<r} T[r][k] in[k], r < n, in slices: lane l of warps 1 and 2 every second term of row l, of warps
+  // 3..7 every fifth of row l + 32.  A float64 instruction takes its warp 64 clocks of its scheduler's unit
+  // whatever its lanes do, so the products run with a row per lane and without warp sums: 97 warp
+  // instructions at 64 columns, where a warp per row and transposed sums took 210.
+  __device__ void lower_slices(const double* in, int n) {
+    static_assert(NW == 8 && MMAX == 64, "two warps for rows 0..31, five for rows 32..63");
+    const bool low = warp <= 2;
+    const int r = low ? lane : lane + 32, st = low ? 2 : 5;
+    double a = 0.0;
+    if (r < n)
+      for (int k = low ? warp - 1 : warp - 3; k < r; k += st) a = fma(small[r * TS + k], in[k], a);
+    part(warp)[lane] = a;
+  }
+  // in[r] plus the slices of row r, in a fixed order.
+  __device__ __forceinline__ double lower_row(const double* in, int r) const {
+    double a = in[r];
+    if (r < 32) a += part(1)[r] + part(2)[r];
+    else a += ((part(3)[r - 32] + part(4)[r - 32]) + (part(5)[r - 32] + part(6)[r - 32])) + part(7)[r - 32];
+    return a;
+  }
+
+  // Strictly lower L = tril(V^T V): cached, above the diagonal of `small`.
+  __device__ __forceinline__ double& Lm(int k, int r) { return cached ? small[r * TS + k] : small[k * TS + r]; }
+
+  // Alg. 7: y = M^{-1} t2; p = (I + N M^{-1}) t2 = t2 - L^T y; H_{1:j,j} solves (I + L) x = p.
+  __device__ void gauss_seidel(int j, const double* temp1, const double* temp2, double* y, double* x) {
+    const int np = j - 1;
+    for (int k = tid; k < np; k += NT) Lm(np, k) = temp1[k];
+    __syncthreads();
+    {                                         // slices as in trow_slices
+      const int r = (warp & 1) * 32 + lane;
+      double acc = 0.0;
+      if (r < j)
+        for (int k = r + 1 + (warp >> 1); k < j; k += 4) acc = fma(Lm(k, r), y[k], acc);
+      part(warp)[lane] = acc;
+    }
+    __syncthreads();
+    for (int r = tid; r < j; r += NT) {
+      const int o = r >> 5, l = r & 31;
+      x[r] = temp2[r] - ((part(o)[l] + part(o + 2)[l]) + (part(o + 4)[l] + part(o + 6)[l]));
+    }
+    __syncthreads();
+    if (warp == 0) {                          // forward substitution, column by column: lane l holds rows l, l + 32
+      double a0 = lane < j ? x[lane] : 0.0, a1 = lane + 32 < j ? x[lane + 32] : 0.0;
+      for (int r = 0; r < j; ++r) {
+        const double l0 = (lane > r && lane < j) ? Lm(lane, r) : 0.0;
+        const double l1 = (lane + 32 > r && lane + 32 < j) ? Lm(lane + 32, r) : 0.0;
+        const double xr = __shfl_sync(0xffffffffu, r < 32 ? a0 : a1, r & 31);
+        a0 = fma(-l0, xr, a0);
+        a1 = fma(-l1, xr, a1);
+      }
+      if (lane < j) x[lane] = a0;
+      if (lane + 32 < j) x[lane + 32] = a1;
+    }
+  }
+
+  // Row `trow` of T from the last step's temp1 (Alg. 5: T_{j,1:j-1} =
+  // -temp_{1:j-1,1}^T T_{1:j-1,1:j-1}; Alg. 6: -temp_{1:j-1,1}^T; for Alg. 7
+  // M^{-1}, as Alg. 5): warps 2s and 2s + 1 take every fourth term, a column
+  // per lane; then the slices are added in a fixed order.
+  __device__ void trow_slices() {
+    const int np = trow, k = (warp & 1) * 32 + lane;
+    const double* temp1 = S.tmp[0];
+    double a = 0.0;
+    if (k < np && P.variant != LSA_HNCWY)
+      for (int i = k + 1 + (warp >> 1); i < np; i += 4) a = fma(temp1[i], small[i * TS + k], a);
+    part(warp)[lane] = a;
+  }
+  __device__ void trow_finish() {
+    const int np = trow;
+    for (int k = tid; k < np; k += NT) {
+      const int o = k >> 5, l = k & 31;
+      const double a = ((part(o)[l] + part(o + 2)[l]) + (part(o + 4)[l] + part(o + 6)[l])) + S.tmp[0][k];
+      small[np * TS + k] = -a;
+    }
+    trow = 0;
+  }
+
+  // The same step in another order of its sums: the float32 form, and the TMA-staged and streaming kernels
+  // (not cached: run by the CTA that completes the reduction).  A coefficient that rounds the other way to
+  // float32 moves a column by 6e-8, so the float32 form keeps one order of the step's sums.
+  __device__ void hybrid_step_ordered(int j) {
+    Ctl* ctl = P.ctl;
+    const int np = j - 1;
+    double* temp1 = S.tmp[0];
+    double* temp2 = S.tmp[1];
+    double* hcol = S.tmp[2];
+    double* aux = S.tmp[3];
+    if (tid == 0) {
+      double Gj = S.red[2 * np], Pj = S.red[2 * np + 1], Q = S.red[2 * np + 2];
+      S.flag = 0;
+      const int syncs = ++S.syncs_c;
+      if (lead) ctl->syncs = syncs;
+      if (j == 1 && Gj == 0.0) {              // zero start vector: y = 0
+        S.flag = 1;
+        if (lead) { ctl->beta = 0.0; ctl->m_eff = 0; ctl->done = 1; }
+      } else if (!(Gj > 0.0) || !isfinite(Gj) || !isfinite(Pj) || !isfinite(Q)) {
+        S.flag = 1;
+        if (lead) { ctl->status = (int)LSA_ERR_NUMERIC; ctl->done = 1; ctl->m_eff = j - 1; }
       } else {
         // one reciprocal square root for both 1/||x|| and ||x|| (a float64
         // warp instruction is slow on this GPU, and this thread is the
@@ -762,27 +1136,21 @@ struct Engine {
         const double nx = Gj * sj;
         S.sj = sj;
         if (j == 1) {
-          ctl->beta = nx;
+          if (lead) ctl->beta = nx;
         } else {
-          const double ne_prev = S.nrm_est_c;
-          const double aw_prev = S.aw_prev_c;
-          double tn = ne_prev * nx;                        // true norm of the previous vector
-          S.true_nrm = tn;
-          if (!(tn > P.brk_tol * aw_prev)) {               // lagged breakdown test
-            Hat(j - 1, j - 2) = tn;
-            ctl->m_eff = j - 1;
-            ctl->breakdown = 1;
-            ctl->done = 1;
+          const double tn = S.nrm_est_c * nx;              // true norm of the previous vector
+          if (lead) Hat(j - 1, j - 2) = tn;
+          if (!(tn > P.brk_tol * S.aw_prev_c)) {           // lagged breakdown test
             S.flag = 1;
+            if (lead) { ctl->m_eff = j - 1; ctl->breakdown = 1; ctl->done = 1; }
           }
         }
-        ctl->sigma[j - 1] = sj;
+        if (lead) ctl->sigma[j - 1] = sj;
         S.sig[j - 1] = sj;
         temp2[np] = sj * sj * Pj;
         temp2[np + 1] = sj * sj * Q;
       }
-      ctl->syncs = ++S.syncs_c;
-      if (cached && S.flag) S.done = 1;
+      if (S.flag) S.done = 1;
     }
     __syncthreads();
     if (S.flag) return;
@@ -797,7 +1165,7 @@ struct Engine {
     } else {
       // New row of T (Alg. 5: T_{j,1:j-1} = -temp_{1:j-1,1}^T T_{1:j-1,1:j-1};
       // Alg. 6: T_{j,1:j-1} = -temp_{1:j-1,1}^T; for Alg. 7 this is M^{-1}).
-      if (!cached && !tcache) stage(P.T, np);   // else small already holds rows 0..np-1 of T
+      if (!cached) stage(P.T, np);              // else small already holds rows 0..np-1 of T
       if (P.variant != LSA_HNCWY) {
         // T_{j,k} = -temp1_k - sum_{i>k} temp1_i T_{i,k}: the four lanes
         // 4k..4k+3 (all eight warps) take the terms i = k+1+q, k+5+q, ...
@@ -806,18 +1174,18 @@ struct Engine {
         const int k = tid >> 2, q = tid & 3;
         double a = 0.0;
         if (k < np)
-          for (int i = k + 1 + q; i < np; i += 4) a = fma(-temp1[i], small[i * MMAX + k], a);
+          for (int i = k + 1 + q; i < np; i += 4) a = fma(-temp1[i], small[i * TS + k], a);
         a += __shfl_xor_sync(0xffffffffu, a, 1);
         a += __shfl_xor_sync(0xffffffffu, a, 2);
         if (k < np && q == 0) {
           const double acc = -temp1[k] + a;
-          small[np * MMAX + k] = acc;
-          P.T[np * MMAX + k] = acc;
+          small[np * TS + k] = acc;
+          if (!cached) P.T[np * MMAX + k] = acc;
         }
       } else {
         for (int k = tid; k < np; k += NT) {
-          small[np * MMAX + k] = -temp1[k];
-          P.T[np * MMAX + k] = -temp1[k];
+          small[np * TS + k] = -temp1[k];
+          if (!cached) P.T[np * MMAX + k] = -temp1[k];
         }
       }
       __syncthreads();
@@ -827,23 +1195,22 @@ struct Engine {
         // Alg. 7: y = M^{-1} temp2; p = (I + N M^{-1}) temp2 = temp2 - L^T y;
         // H_{1:j,j} solves (I + L) x = p.
         apply_unit_lower(temp2, aux, j);                  // aux = y
-        double* Lm = cached ? smallL : small;             // L (cached: kept between steps)
         if (!cached) stage(P.L, np);
         for (int k = tid; k < np; k += NT) {
-          Lm[np * MMAX + k] = temp1[k];
-          P.L[np * MMAX + k] = temp1[k];
+          Lm(np, k) = temp1[k];
+          if (!cached) P.L[np * MMAX + k] = temp1[k];
         }
         __syncthreads();
         for (int r = tid; r < j; r += NT) {
           double acc = 0.0;
-          for (int k = r + 1; k < j; ++k) acc = fma(Lm[k * MMAX + r], aux[k], acc);
+          for (int k = r + 1; k < j; ++k) acc = fma(Lm(k, r), aux[k], acc);
           hcol[r] = temp2[r] - acc;
         }
         __syncthreads();
         if (warp == 0) {                                   // forward substitution
           for (int r = 0; r < j; ++r) {
             double acc = 0.0;
-            for (int k = lane; k < r; k += 32) acc = fma(Lm[r * MMAX + k], hcol[k], acc);
+            for (int k = lane; k < r; k += 32) acc = fma(Lm(r, k), hcol[k], acc);
             acc = warp_sum(acc);
             if (lane == 0) hcol[r] = hcol[r] - acc;
             __syncwarp();
@@ -852,56 +1219,51 @@ struct Engine {
       }
     }
     __syncthreads();
-    for (int r = tid; r < j; r += NT) Hat(r, j - 1) = hcol[r];
+    if (lead)
+      for (int r = tid; r < j; r += NT) Hat(r, j - 1) = hcol[r];
     if (warp == 0) {
       double ss = 0.0;
       for (int i = lane; i < j; i += 32) ss = fma(temp2[i], temp2[i], ss);
       ss = warp_sum(ss);
-      if (lane == 0) S.ss = ss;
+      if (lane == 0) part(0)[0] = ss;
     }
     __syncthreads();
     if (tid == 0) {
-      if (j > 1) Hat(j - 1, j - 2) = S.true_nrm;
-      double t = temp2[j];
-      double awn = sqrt(t);
-      S.scale = 1.0;
+      const double ss = part(0)[0], t = temp2[j];
+      const double awn = sqrt(t);
+      double ne = 1.0, scale = 1.0;
       bool done_now = false;
-      if (t < S.ss) {                         // Pythagorean radicand negative: explicit norm
-        ctl->fallbacks = __ldcg(&ctl->fallbacks) + 1;
-        ctl->fallback_pending = 1;
-        ctl->nrm_est = 1.0;
-        S.nrm_est_c = 1.0;
-        if (cached) S.fallback_pending = 1;
+      if (t < ss) {                           // Pythagorean radicand negative: explicit norm
+        if (lead) { atomicAdd(&ctl->fallbacks, 1); ctl->fallback_pending = 1; }
+        S.fallback_pending = 1;
       } else {
-        const double d = t - S.ss;            // Eq. 18: ne = sqrt(d), scale = 1/ne
+        const double d = t - ss;              // Eq. 18: ne = sqrt(d), scale = 1/ne
         const double rd = (d > 0.0) ? rsqrt(d) : 0.0;
-        const double ne = d * rd;
+        ne = d * rd;
+        scale = rd;
         if (!(ne > P.brk_tol * awn)) {
-          Hat(j, j - 1) = ne;
-          ctl->m_eff = j;
-          ctl->breakdown = 1;
-          ctl->done = 1;
+          if (lead) { Hat(j, j - 1) = ne; ctl->m_eff = j; ctl->breakdown = 1; ctl->done = 1; }
+          S.done = 1;
           done_now = true;
         }
-        ctl->nrm_est = ne;
-        S.nrm_est_c = ne;
-        S.scale = rd;
       }
-      ctl->aw_prev = awn;
+      S.scale = scale;
+      S.nrm_est_c = ne;
       S.aw_prev_c = awn;
-      ctl->a = S.sj * S.scale;
-      if (cached) {
-        S.a = (Tc)(S.sj * S.scale);
-        if (done_now) S.done = 1;
+      S.a = (Tc)(S.sj * scale);
+      if (lead) {
+        ctl->nrm_est = ne;
+        ctl->aw_prev = awn;
+        ctl->a = S.sj * scale;
+        if (j == P.m && !done_now) ctl->m_eff = P.m;
       }
-      if (j == P.m && !done_now && !__ldcg(&ctl->done)) ctl->m_eff = P.m;
     }
     __syncthreads();
     for (int i = tid; i < j; i += NT) {
       double si = (i == j - 1) ? S.sj : S.sig[i];
       const double c = si * hcol[i] * S.scale;
-      ctl->coef[i] = c;
       if (cached) S.coefc[i] = (Tc)c;
+      else ctl->coef[i] = c;
     }
   }
 
@@ -923,7 +1285,7 @@ struct Engine {
       for (int u = 0; u < U; ++u) {
         const int e = e0 + u * NT;
         const int r = e / MMAX, k = e - r * MMAX;
-        if (e < total && k < r) small[e] = v[u];
+        if (e < total && k < r) small[r * TS + k] = v[u];
       }
     }
     __syncthreads();
@@ -939,7 +1301,7 @@ struct Engine {
       const int r = warp + NW * i;
       double a = 0.0;
       if (r < n)
-        for (int k = lane; k < r; k += 32) a = fma(small[r * MMAX + k], in[k], a);
+        for (int k = lane; k < r; k += 32) a = fma(small[r * TS + k], in[k], a);
       acc[i] = a;
     }
     const double sum = warp_sum_many<8>(acc);   // lane l: row warp + NW*(l >> 2)
@@ -952,32 +1314,33 @@ struct Engine {
     Ctl* ctl = P.ctl;
     if (tid == 0) {
       double nrm = sqrt(S.red[0]);
-      ctl->syncs = ++S.syncs_c;
+      const int syncs = ++S.syncs_c;
       if (!(nrm > P.brk_tol * S.aw_prev_c)) {
-        Hat(j, j - 1) = nrm;
-        ctl->m_eff = j;
-        ctl->breakdown = 1;
-        ctl->done = 1;
-        if (cached) S.done = 1;
+        if (lead) { Hat(j, j - 1) = nrm; ctl->m_eff = j; ctl->breakdown = 1; ctl->done = 1; }
+        S.done = 1;
       }
-      ctl->nrm_est = nrm;
       S.nrm_est_c = nrm;
       S.scale = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      ctl->a = (cached ? (double)S.a : __ldcg(&ctl->a)) * S.scale;
-      ctl->fallback_pending = 0;
-      if (cached) { S.a = (Tc)(S.a * S.scale); S.fallback_pending = 0; }
+      const double a = (cached ? S.sj : __ldcg(&ctl->a)) * S.scale;   // (the step left scale 1)
+      S.a = (Tc)a;
+      S.fallback_pending = 0;
+      if (lead) {
+        ctl->syncs = syncs;
+        ctl->nrm_est = nrm;
+        ctl->a = a;
+        ctl->fallback_pending = 0;
+      }
     }
     __syncthreads();
     for (int i = tid; i < j; i += NT) {
-      const double c = (cached ? (double)S.coefc[i] : __ldcg(&ctl->coef[i])) * S.scale;
-      ctl->coef[i] = c;
-      if (cached) S.coefc[i] = (Tc)c;
+      if (cached) S.coefc[i] = (Tc)(S.sig[i] * S.tmp[2][i] * S.scale);
+      else ctl->coef[i] = __ldcg(&ctl->coef[i]) * S.scale;
     }
   }
 
   __device__ void hybrid_final_finish() {
     Ctl* ctl = P.ctl;
-    if (tid == 0) {
+    if (tid == 0 && lead) {
       const int m = P.m;
       double nrm = sqrt(S.red[0]);
       double hl = S.nrm_est_c * nrm;   // true norm of the projected v_{m+1}
@@ -999,15 +1362,13 @@ struct Engine {
     B* Wb[2] = {reinterpret_cast<B*>(P.W0), reinterpret_cast<B*>(P.W1)};
     const long long N = P.op.N;
     const int m = P.m;
-    unsigned gen = 0;
     if (tid == 0) { S.a = (Tc)1; S.done = 0; S.fallback_pending = 0; S.syncs_c = 0; }
     __syncthreads();
     // Two-phase form: a pass over equal flat shares projects x_j (no halo),
     // a grid barrier, then the tile pass reads x_j back with its halo for
     // w_j = A x_j and the inner products.  Every value goes through the same
     // operations in the same order as in the one-pass form.
-    const bool two = P.two_phase != 0 && !AUG && !cached;
-    tcache = !cached && P.variant != LSA_HGSMGS;
+    const bool two = P.two_phase != 0 && !AUG;
     for (int j = 1; j <= m; ++j) {
       PassT<B> ps;
       ps.c0 = 0; ps.c1 = j - 1;
@@ -1021,7 +1382,7 @@ struct Engine {
       ps.self = SELF_XX | SELF_XW | SELF_WW;
       if (two) {
         project_flat(ps);                      // x_j (no halo)
-        if (!sync_only(gen)) return;
+        if (!sync_only()) return;
         ps.c0 = ps.c1 = 0;                     // then x_j with its halo, w_j = A x_j, the products
         ps.a = 1.0;
         ps.src64 = nullptr;
@@ -1029,7 +1390,7 @@ struct Engine {
         ps.xout = nullptr;
       }
       const int ns = run_pass(ps);
-      if (!reduce_step(gen, ns, j, [&] { hybrid_step(j); }, j - 1)) return;
+      if (!reduce_all(ns, [&] { hybrid_step(j); })) return;
       if (S.done) return;
       if (S.fallback_pending) {
         // explicit norm of the projected vector (extra reduction of Alg. 4)
@@ -1039,7 +1400,7 @@ struct Engine {
         pf.xout = nullptr; pf.wout = nullptr;
         pf.d0 = 0; pf.d1 = 0; pf.dmode = 0; pf.self = SELF_XX;
         int nf = run_pass(pf);
-        if (!reduce_step(gen, nf, j, [&] { hybrid_fallback_finish(j); })) return;
+        if (!reduce_all(nf, [&] { hybrid_fallback_finish(j); })) return;
         if (S.done) return;
       }
     }
@@ -1050,27 +1411,39 @@ struct Engine {
     pl.xout = V + (long long)m * N; pl.wout = nullptr;
     pl.d0 = 0; pl.d1 = 0; pl.dmode = 0; pl.self = SELF_XX;
     int nl = run_pass(pl);
-    reduce_step(gen, nl, 0, [&] { hybrid_final_finish(); });
+    reduce_all(nl, [&] { hybrid_final_finish(); });
   }
 
   // -------------------------------------------------------------------------
   // Shared pieces of MGS and CGS2: ||v|| and the "next vector" pass.
-  __device__ bool norm_of_input(unsigned& gen) {
+  __device__ bool norm_of_input() {
     PassT<B> ps;
     ps.c0 = ps.c1 = 0; ps.a = 1.0; ps.src64 = P.vin; ps.srcB = nullptr;
     ps.xout = nullptr; ps.wout = nullptr; ps.d0 = ps.d1 = 0; ps.dmode = 0; ps.self = SELF_XX;
     int ns = run_pass(ps);
-    return reduce_step(gen, ns, 0, [&] {
+    return reduce_all(ns, [&] {
       if (tid == 0) {
         double b = sqrt(S.red[0]);
-        P.ctl->beta = b;
-        P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1;
-        if (b == 0.0) { P.ctl->done = 1; P.ctl->m_eff = 0; }     // zero start vector: y = 0
-        else if (!isfinite(b)) { P.ctl->done = 1; P.ctl->status = (int)LSA_ERR_NUMERIC; }
-        P.ctl->a = (b > 0.0) ? 1.0 / b : 0.0;
-        for (int i = 0; i <= P.m; ++i) P.ctl->sigma[i] = 1.0;
+        S.syncs_c = 1;
+        S.done = b == 0.0 || !isfinite(b);     // zero start vector: y = 0
+        S.a = (Tc)((b > 0.0) ? 1.0 / b : 0.0);
+        if (lead) {
+          P.ctl->beta = b;
+          P.ctl->syncs = 1;
+          if (S.done) P.ctl->done = 1;
+          if (b == 0.0) P.ctl->m_eff = 0;
+          else if (S.done) P.ctl->status = (int)LSA_ERR_NUMERIC;
+        }
       }
+      if (lead)
+        for (int i = tid; i <= P.m; i += NT) P.ctl->sigma[i] = 1.0;
     });
+  }
+
+  // One more reduction of a step (thread 0).
+  __device__ __forceinline__ void count_sync() {
+    const int n = ++S.syncs_c;
+    if (lead) P.ctl->syncs = n;
   }
 
   // write v_{m+1} = a * w (no reduction): only for the Arnoldi output
@@ -1087,8 +1460,7 @@ struct Engine {
     B* Wb[2] = {reinterpret_cast<B*>(P.W0), reinterpret_cast<B*>(P.W1)};
     const long long N = P.op.N;
     const int m = P.m;
-    unsigned gen = 0;
-    if (!norm_of_input(gen)) return;
+    if (!norm_of_input()) return;
     if (S.done) return;
     for (int j = 1; j <= m; ++j) {
       B* w = Wb[j & 1];
@@ -1101,15 +1473,15 @@ struct Engine {
       pa.d0 = 0; pa.d1 = (j > 1) ? 1 : 0; pa.dmode = DOT_W;
       pa.self = SELF_XW | SELF_WW;
       int ns = run_pass(pa);
-      if (!reduce_step(gen, ns, 1, [&] {
+      if (!reduce_all(ns, [&] {
             if (tid == 0) {
               const int nd = (j > 1) ? 1 : 0;
               // H_{1,j} = v_1 . w: the W slot of column 0, or x.w when v_1 = x
               double h = (j > 1) ? S.red[nd] : S.red[2 * nd + 1];
-              Hat(0, j - 1) = h;
-              P.ctl->coef[0] = h;
-              P.ctl->aw_prev = sqrt(S.red[2 * nd + 2]);
-              P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1;
+              if (lead) Hat(0, j - 1) = h;
+              S.coefc[0] = (Tc)h;
+              S.aw_prev_c = sqrt(S.red[2 * nd + 2]);
+              count_sync();
             }
           })) return;
       for (int i = 1; i < j; ++i) {
@@ -1119,12 +1491,12 @@ struct Engine {
         pu.xout = w; pu.wout = nullptr;
         pu.d0 = i; pu.d1 = i + 1; pu.dmode = DOT_X; pu.self = 0;
         int nu = run_pass(pu);
-        if (!reduce_step(gen, nu, i + 1, [&] {
+        if (!reduce_all(nu, [&] {
               if (tid == 0) {
                 double h = S.red[0];
-                Hat(i, j - 1) = h;
-                P.ctl->coef[i] = h;
-                P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1;
+                if (lead) Hat(i, j - 1) = h;
+                S.coefc[i] = (Tc)h;
+                count_sync();
               }
             })) return;
       }
@@ -1133,7 +1505,7 @@ struct Engine {
       pz.c0 = j - 1; pz.c1 = j; pz.a = 1.0; pz.src64 = nullptr; pz.srcB = w;
       pz.xout = w; pz.wout = nullptr; pz.d0 = pz.d1 = 0; pz.dmode = 0; pz.self = SELF_XX;
       int nz = run_pass(pz);
-      if (!reduce_step(gen, nz, 0, [&] { finish_norm(j); })) return;
+      if (!reduce_all(nz, [&] { finish_norm(j); })) return;
       if (S.done) return;
     }
     if (write_vlast) write_last(V + (long long)m * N, Wb[m & 1]);
@@ -1143,17 +1515,17 @@ struct Engine {
     if (tid == 0) {
       Ctl* ctl = P.ctl;
       double nrm = sqrt(S.red[0]);
-      Hat(j, j - 1) = nrm;
-      ctl->syncs = cached ? ++S.syncs_c : __ldcg(&ctl->syncs) + 1;
-      if (!(nrm > P.brk_tol * __ldcg(&ctl->aw_prev))) {
-        ctl->m_eff = j;
-        ctl->breakdown = 1;
-        ctl->done = 1;
+      count_sync();
+      const bool brk = !(nrm > P.brk_tol * S.aw_prev_c), bad = !isfinite(nrm);
+      S.done = brk || bad;
+      S.a = (Tc)((nrm > 0.0) ? 1.0 / nrm : 0.0);
+      if (lead) {
+        Hat(j, j - 1) = nrm;
+        if (brk) { ctl->m_eff = j; ctl->breakdown = 1; ctl->done = 1; }
+        if (bad) { ctl->status = (int)LSA_ERR_NUMERIC; ctl->done = 1; ctl->m_eff = j - 1; }
+        ctl->h_last = nrm;
+        if (j == P.m && !S.done) ctl->m_eff = P.m;
       }
-      if (!isfinite(nrm)) { ctl->status = (int)LSA_ERR_NUMERIC; ctl->done = 1; ctl->m_eff = j - 1; }
-      ctl->a = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      ctl->h_last = nrm;
-      if (j == P.m && !__ldcg(&ctl->done)) ctl->m_eff = P.m;
     }
   }
 
@@ -1163,8 +1535,7 @@ struct Engine {
     B* Wb[2] = {reinterpret_cast<B*>(P.W0), reinterpret_cast<B*>(P.W1)};
     const long long N = P.op.N;
     const int m = P.m;
-    unsigned gen = 0;
-    if (!norm_of_input(gen)) return;
+    if (!norm_of_input()) return;
     if (S.done) return;
     for (int j = 1; j <= m; ++j) {
       B* w = Wb[j & 1];
@@ -1176,32 +1547,32 @@ struct Engine {
       pa.d0 = 0; pa.d1 = j - 1; pa.dmode = DOT_W;
       pa.self = SELF_XW | SELF_WW;
       int ns = run_pass(pa);
-      if (!reduce_step(gen, ns, j, [&] {
+      if (!reduce_all(ns, [&] {
             const int nd = j - 1;
             for (int i = tid; i < j; i += NT) {
               double h = (i < nd) ? S.red[nd + i] : S.red[2 * nd + 1];
-              P.ctl->hcol[i] = h;
-              P.ctl->coef[i] = h;
+              S.tmp[2][i] = h;
+              S.coefc[i] = (Tc)h;
             }
-            if (tid == 0) { P.ctl->aw_prev = sqrt(S.red[2 * nd + 2]); P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1; }
+            if (tid == 0) { S.aw_prev_c = sqrt(S.red[2 * nd + 2]); count_sync(); }
           })) return;
       PassT<B> pb;
       pb.c0 = 0; pb.c1 = j; pb.a = 1.0; pb.src64 = nullptr; pb.srcB = w;
       pb.xout = w; pb.wout = nullptr; pb.d0 = 0; pb.d1 = j; pb.dmode = DOT_X; pb.self = 0;
       int nb = run_pass(pb);
-      if (!reduce_step(gen, nb, j, [&] {
+      if (!reduce_all(nb, [&] {
             for (int i = tid; i < j; i += NT) {
               double h2 = S.red[i];
-              Hat(i, j - 1) = __ldcg(&P.ctl->hcol[i]) + h2;
-              P.ctl->coef[i] = h2;
+              if (lead) Hat(i, j - 1) = S.tmp[2][i] + h2;
+              S.coefc[i] = (Tc)h2;
             }
-            if (tid == 0) P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1;
+            if (tid == 0) count_sync();
           })) return;
       PassT<B> pc;
       pc.c0 = 0; pc.c1 = j; pc.a = 1.0; pc.src64 = nullptr; pc.srcB = w;
       pc.xout = w; pc.wout = nullptr; pc.d0 = pc.d1 = 0; pc.dmode = 0; pc.self = SELF_XX;
       int nc = run_pass(pc);
-      if (!reduce_step(gen, nc, 0, [&] { finish_norm(j); })) return;
+      if (!reduce_all(nc, [&] { finish_norm(j); })) return;
       if (S.done) return;
     }
     if (write_vlast) write_last(V + (long long)m * N, Wb[m & 1]);
@@ -1215,8 +1586,7 @@ struct Engine {
     B* Wb[2] = {reinterpret_cast<B*>(P.W0), reinterpret_cast<B*>(P.W1)};
     const long long N = P.op.N;
     const int m = P.m;
-    unsigned gen = 0;
-    if (!norm_of_input(gen)) return;
+    if (!norm_of_input()) return;
     if (S.done) return;
     for (int j = 1; j <= m; ++j) {
       B* w = Wb[j & 1];
@@ -1230,21 +1600,21 @@ struct Engine {
       pa.d0 = lo; pa.d1 = j - 1; pa.dmode = DOT_W;
       pa.self = SELF_XW | SELF_WW;
       int ns = run_pass(pa);
-      if (!reduce_step(gen, ns, j, [&] {
+      if (!reduce_all(ns, [&] {
             const int nd = j - 1 - lo;
             for (int i = lo + tid; i < j; i += NT) {
               double h = (i < j - 1) ? S.red[nd + i - lo] : S.red[2 * nd + 1];
-              Hat(i, j - 1) = h;
-              P.ctl->coef[i] = h;
+              if (lead) Hat(i, j - 1) = h;
+              S.coefc[i] = (Tc)h;
             }
-            if (tid == 0) { P.ctl->aw_prev = sqrt(S.red[2 * nd + 2]); P.ctl->syncs = __ldcg(&P.ctl->syncs) + 1; }
+            if (tid == 0) { S.aw_prev_c = sqrt(S.red[2 * nd + 2]); count_sync(); }
           })) return;
       // w -= H_{lo..j,j} v_{lo..j}; ||w||
       PassT<B> pc;
       pc.c0 = lo; pc.c1 = j; pc.a = 1.0; pc.src64 = nullptr; pc.srcB = w;
       pc.xout = w; pc.wout = nullptr; pc.d0 = pc.d1 = 0; pc.dmode = 0; pc.self = SELF_XX;
       int nc = run_pass(pc);
-      if (!reduce_step(gen, nc, 0, [&] { finish_norm(j); })) return;
+      if (!reduce_all(nc, [&] { finish_norm(j); })) return;
       if (S.done) return;
     }
     if (write_vlast) write_last(V + (long long)m * N, Wb[m & 1]);
@@ -1266,6 +1636,7 @@ __global__ void __launch_bounds__(NT, (sizeof(Tc) == 8) ? LSA_MINB_F64 : LSA_MIN
   typename E::Smem& S = *reinterpret_cast<typename E::Smem*>(smem_raw);
   E e(P, S, reinterpret_cast<double*>(smem_raw + E::small_offset()));
   if (!e.place()) return;
+  e.redundant_steps();
   if (P.variant == LSA_MGS) e.run_mgs(P.write_vlast != 0);
   else if (P.variant == LSA_CGS2) e.run_cgs2(P.write_vlast != 0);
   else if (P.variant == LSA_IOCGS) e.run_iocgs(P.write_vlast != 0);
@@ -1292,10 +1663,13 @@ cudaError_t launch_arnoldi_t(const ArnoldiParams& P, int G, cudaStream_t s) {
   ArnoldiParams Pc = P;
   void* args[1] = {&Pc};
   auto k = k_arnoldi<Op, Tc, Tc>;
-  if constexpr (sizeof(Tc) == 8 && Op::KIND <= LSA_OP_ADR3D) {   // the three workload operators
-    if (P.naug > 0) k = k_arnoldi<Op, Tc, Tc, true>;
-  }
   size_t sm = Engine<Op, Tc, Tc>::smem_bytes();
+  if constexpr (sizeof(Tc) == 8 && Op::KIND <= LSA_OP_ADR3D) {   // the three workload operators
+    if (P.naug > 0) {
+      k = k_arnoldi<Op, Tc, Tc, true>;
+      sm = Engine<Op, Tc, Tc, true>::smem_bytes();
+    }
+  }
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel((void*)k, dim3(G), dim3(NT), args, sm, s);

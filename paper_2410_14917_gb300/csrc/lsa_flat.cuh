@@ -48,7 +48,7 @@ __device__ __forceinline__ void flat_wait() { asm volatile("cp.async.wait_group 
 
 template <class Op, class Tc, bool AUG = false>
 struct FlatPass {
-  using E = Engine<Op, Tc, Tc, AUG>;
+  using E = Engine<Op, Tc, Tc, AUG, sizeof(Tc) == 4>;   // (float32: the tile passes for its norm passes)
   static constexpr int NS = Op::NS;
   static constexpr bool F64 = sizeof(Tc) == 8;
   static constexpr int VW = F64 ? 2 : 4;                 // values of a 16-byte load
@@ -622,7 +622,7 @@ struct FlatPass {
     }
     warp_sum_many_comp<2 * KMAX>(vs, ve);    // lanes 2k, 2k + 1: value k (column k / 2 of the warp, x or w)
     const int k = e.lane >> 1, c = e.warp + NW * (k >> 1);
-    if ((e.lane & 1) == 0 && c < nd) (e.P.partials + (long long)e.grank * SLOTS)[(k & 1) ? nd + c : c] = (double)vs[0] + (double)ve[0];
+    if ((e.lane & 1) == 0 && c < nd) e.part_row()[(k & 1) ? nd + c : c] = (double)vs[0] + (double)ve[0];
     return e.write_self(ps, nd);
   }
   __device__ int pass(const PassT<Tc>& ps) {
@@ -634,7 +634,7 @@ struct FlatPass {
   // float64: per-CTA partial sums to global memory in the engine's layout: x_i . x and x_i . w of the earlier
   // columns, then x . x, x . w (column nc - 1) and w . w.
   __device__ int partials_fixed(int nc) {
-    double* part = e.P.partials + (long long)e.grank * SLOTS;
+    double* part = e.part_row();
     const int np = nc - 1;
     const double ww = warp_sum(e.sww);
     if (e.lane == 0) e.S.bred[e.warp][2] = ww;
@@ -667,10 +667,8 @@ struct FlatPass {
     Tc* Wb[2] = {reinterpret_cast<Tc*>(P.W0), reinterpret_cast<Tc*>(P.W1)};
     const long long N = P.op.N;
     const int m = P.m;
-    unsigned gen = 0;
     if (e.tid == 0) { e.S.a = (Tc)1; e.S.done = 0; e.S.fallback_pending = 0; e.S.syncs_c = 0; }
     __syncthreads();
-    e.tcache = P.variant != LSA_HGSMGS;
     PassT<Tc> ps;
     ps.dmode = DOT_X | DOT_W;
     for (int j = 1; j <= m; ++j) {
@@ -684,7 +682,7 @@ struct FlatPass {
       ps.self = 0;
       if constexpr (AUG) e.aug_begin(ps);
       project(ps, j - 1);
-      if (!e.sync_only(gen)) return;
+      if (!e.sync_only()) return;
       ps.c0 = ps.c1 = 0;
       ps.a = 1.0;
       ps.src64 = nullptr;
@@ -693,29 +691,29 @@ struct FlatPass {
       ps.d1 = F64 ? j : j - 1;         // float64: the last column is x_j itself
       ps.self = F64 ? SELF_WW : SELF_XX | SELF_XW | SELF_WW;
       const int ns = pass(ps);
-      if (!e.reduce_step(gen, ns, j, [&] { e.hybrid_step(j); }, j - 1)) return;
+      if (!e.reduce_all(ns, [&] { e.hybrid_step(j); })) return;
       if (e.S.done) return;
       if (e.S.fallback_pending) {     // explicit norm of the projected vector (extra reduction of Alg. 4)
-        if (!norm_pass(gen, j, Wb[j & 1], nullptr, [&] { e.hybrid_fallback_finish(j); }, j)) return;
+        if (!norm_pass(j, Wb[j & 1], nullptr, [&] { e.hybrid_fallback_finish(j); })) return;
         if (e.S.done) return;
       }
     }
     // v_{m+1} and its norm (one more reduction)
-    norm_pass(gen, m, Wb[m & 1], V + (long long)m * N, [&] { e.hybrid_final_finish(); }, 0);
+    norm_pass(m, Wb[m & 1], V + (long long)m * N, [&] { e.hybrid_final_finish(); });
   }
 
   // x = a src - sum_{c < nc} coef_c V_c and x . x, reduced; x stored when xout is given.
   template <class Fn>
-  __device__ bool norm_pass(unsigned& gen, int nc, const Tc* src, Tc* xout, Fn fn, int ncoef) {
+  __device__ bool norm_pass(int nc, const Tc* src, Tc* xout, Fn fn) {
     PassT<Tc> ps;
     ps.c0 = 0; ps.c1 = nc; ps.a = (double)e.S.a;
     ps.src64 = nullptr; ps.srcB = src; ps.xout = xout; ps.wout = nullptr;
     ps.d0 = ps.d1 = 0; ps.dmode = 0; ps.self = SELF_XX;
-    if constexpr (!F64) return e.reduce_step(gen, e.run_pass(ps), ncoef, fn);
+    if constexpr (!F64) return e.reduce_all(e.run_pass(ps), fn);
     e.zero_acc();
     if constexpr (AUG) e.aug_begin(ps);
     project(ps, -1);
-    return e.reduce_step(gen, e.write_self(ps, 0), ncoef, fn);
+    return e.reduce_all(e.write_self(ps, 0), fn);
   }
 };
 
@@ -727,6 +725,7 @@ __global__ void __launch_bounds__(NT, 2) k_arnoldi_flat(ArnoldiParams P) {
   typename E::Smem& S = *reinterpret_cast<typename E::Smem*>(smem_raw);
   E e(P, S, reinterpret_cast<double*>(smem_raw + E::small_offset()));
   if (!e.place()) return;
+  e.redundant_steps();
   F f(e, *reinterpret_cast<typename F::Buf*>(smem_raw + F::offset()));
   f.run();
 }

@@ -10,6 +10,8 @@ namespace lsa {
 
 constexpr int MMAX = 64;                  // largest Krylov dimension of the fused kernels
 constexpr int PMAX = 8;                   // largest phi index p
+constexpr int TS = MMAX + 1;              // row stride of T in shared memory (odd: rows and columns without bank conflicts)
+constexpr int STEP_DOUBLES = MMAX * TS + (256 / 32) * 32;   // scratch of the O(j^2) step: T and the slices of its products
 constexpr int SLOTS = 2 * MMAX + 4;       // reduction slots per CTA and pass
 constexpr int NT = 256;                   // threads per CTA of the Arnoldi kernels
 constexpr int NW = NT / 32;
@@ -92,7 +94,8 @@ struct ArnoldiParams {
   double* H;               // (m+1) x m column-major, leading dimension m+1
   Ctl* ctl;
   double* partials;        // gridDim.x x SLOTS
-  double* gsum;            // two-level reduction: per-group sums, RG_MAX x SLOTS (null: one level)
+  double* gsum;            // RG_MAX x SLOTS: the reduced sums, or a small grid's second buffer of partial sums
+                           // (TMA-staged and streaming kernels: sums per group of RG CTAs)
   double* T;               // MMAX x MMAX correction matrix (CWY/NCWY T, GSMGS M^{-1})
   double* L;               // MMAX x MMAX strictly lower part of V^T V (GSMGS)
   int m;
@@ -109,13 +112,12 @@ struct ArnoldiParams {
   // with B = [b_p, ..., b_1] and K the p x p upper shift.  naug = 0: plain A.
   int naug;
   const double* baug;      // b_0..b_p, (p+1) x N (column k of B is b_{p-k})
-  double* xaug;            // extra entries of the extended basis columns, (m+3) x PMAX
   double aug_t;            // extra entries of the start vector: exp(aug_t K) e_p
 };
 
 // Workspace layout (all offsets 256-byte aligned).
 struct Layout {
-  size_t ctl, partials, gsum, T, L, H, V, W0, W1, small, coefs, g0, g1, E, F, xaug;
+  size_t ctl, partials, gsum, T, L, H, V, W0, W1, small, coefs, g0, g1, E, F;
   size_t base, total;      // without and with the limbs F
   int G;                   // CTAs of the persistent Arnoldi kernel
 };

@@ -774,7 +774,7 @@ bool stream_applicable_op(const DevOp& d, const Tiling& tl, int m) {
   const int s_hyb = stream_stage_bytes(m - 1, Op::NF > 0 ? 1 : 0);
   const int s_fin = stream_stage_bytes(m, 0);
   if (cap / s_hyb < 2 + lag || cap / s_fin < 2) return false;
-  return cap >= (int)(sizeof(double) * MMAX * MMAX) && cap >= (int)(sizeof(double) * 2 * NW * MMAX);
+  return cap >= (int)(sizeof(double) * STEP_DOUBLES) && cap >= (int)(sizeof(double) * 2 * NW * MMAX);
 }
 
 template <class Op>

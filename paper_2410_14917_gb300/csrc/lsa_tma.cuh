@@ -132,7 +132,7 @@ struct TmaLayout {
   }
   static __host__ __device__ size_t smem_bytes(int ncap) {
     size_t st = (size_t)3 * stage_bytes(ncap);
-    size_t mn = sizeof(double) * MMAX * MMAX;             // the last CTA's scratch aliases the stages
+    size_t mn = sizeof(double) * STEP_DOUBLES;             // the last CTA's scratch aliases the stages
     return head_bytes() + (st > mn ? st : mn);
   }
   static __host__ __device__ int ncap_for(int m) { return (m + 1) & ~1; }   // even, >= m
