@@ -1,6 +1,5 @@
 // Arnoldi kernels instantiated for the adr3d operator (one translation unit
 // per operator so that the library builds in parallel).
-#include "lsa_batched.cuh"
 #include "lsa_stream.cuh"
 #include "lsa_tma.cuh"
 
@@ -29,10 +28,5 @@ bool stream_applicable_adr3d(const DevOp& d, const Tiling& tl, int m) {
 cudaError_t launch_arnoldi_stream_adr3d(const ArnoldiParams& P, cudaStream_t s) {
   return launch_arnoldi_stream_op<OpADR3D>(P, s);
 }
-
-cudaError_t launch_batched_adr3d(const BatchParams& BP, int precision, int G, cudaStream_t s) {
-  return launch_batched_op<OpADR3D>(BP, precision, G, s);
-}
-int batched_blocks_per_sm_adr3d(int precision) { return batched_blocks_per_sm_op<OpADR3D>(precision); }
 
 }  // namespace lsa

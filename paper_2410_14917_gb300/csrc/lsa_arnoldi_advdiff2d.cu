@@ -1,6 +1,5 @@
 // Arnoldi kernels instantiated for the advdiff2d operator (one translation unit
 // per operator so that the library builds in parallel).
-#include "lsa_batched.cuh"
 #include "lsa_cluster.cuh"
 #include "lsa_stream.cuh"
 #include "lsa_tma.cuh"
@@ -38,10 +37,5 @@ cudaError_t launch_arnoldi_cluster_advdiff2d(const ArnoldiParams& P, const Small
                                              cudaStream_t s) {
   return launch_arnoldi_cluster_op<OpAdvDiff2D>(P, SP, y, s);
 }
-
-cudaError_t launch_batched_advdiff2d(const BatchParams& BP, int precision, int G, cudaStream_t s) {
-  return launch_batched_op<OpAdvDiff2D>(BP, precision, G, s);
-}
-int batched_blocks_per_sm_advdiff2d(int precision) { return batched_blocks_per_sm_op<OpAdvDiff2D>(precision); }
 
 }  // namespace lsa

@@ -77,7 +77,8 @@ struct BatchLayout {
   int G = 0, count = 0;
   size_t bctl = 0, mail = 0, inst = 0, order = 0, partials = 0, T = 0, L = 0, mats = 0;
   size_t ctl = 0, ctl_stride = 0, total = 0;
-  std::vector<size_t> H, C, V, g0, g1;
+  std::vector<size_t> H, C, V, g0, g1, F;
+  bool limbs = false;
   std::vector<DevOp> d;
   std::vector<int> m;
 };
@@ -133,6 +134,15 @@ static lsa_status batch_layout(const lsa_op* ops, const int* ms, int count, int 
     BL->g0[i] = take(nfield * sizeof(float));
     BL->g1[i] = take(nfield * sizeof(float));
   }
+
+  BL->F.resize(count);
+  BL->limbs = false;
+  if (precision == LSA_FP64) {
+    size_t bytes = 0;
+    for (int i = 0; i < count; ++i) bytes += align256(limb_bytes(BL->d[i], BL->m[i]));
+    BL->limbs = bytes <= kLimbBytes;
+    for (int i = 0; i < count && BL->limbs; ++i) BL->F[i] = take(limb_bytes(BL->d[i], BL->m[i]));
+  }
   BL->total = off;
   return LSA_OK;
 }
@@ -146,7 +156,7 @@ struct lsa_batch {
   double h = 0.0, tol = 0.0;
   int G = 0;
   int gsize = 1, nlarge = 0;
-  int two_phase = 0;                 // step form of the hybrid variants
+  int step = 0;                      // step form of the hybrid variants (BatchParams::step)
   char* w = nullptr;
   BatchLayout BL;
   std::vector<BatchInst> inst;
@@ -168,7 +178,7 @@ struct lsa_batch {
     BP.count = count;
     BP.nlarge = nlarge;
     BP.gsize = gsize;
-    BP.two_phase = two_phase;
+    BP.step = step;
     BP.variant = variant;
     BP.p = p;
     BP.h = h;
@@ -264,6 +274,7 @@ lsa_status lsa_batch_create(const lsa_op* ops, const int* m, int count, double h
     I.H = (double*)(b->w + b->BL.H[i]);
     I.C = (double*)(b->w + b->BL.C[i]);
     I.V = b->w + b->BL.V[i];
+    I.F = b->BL.limbs ? (int2*)(b->w + b->BL.F[i]) : nullptr;
     b->voff[i] = nv;
     b->yoff[i] = ny;
     nv += I.op.N;
@@ -289,9 +300,9 @@ lsa_status lsa_batch_create(const lsa_op* ops, const int* m, int count, double h
   b->nlarge = nl;
   if (b->nlarge == 0) b->gsize = 1;
   // default step form of the hybrid variants: two-phase (its barrier between
-  // the passes counts only an instance's group; faster in both precisions on
-  // the 512-instance advection-diffusion batch)
-  b->two_phase = is_hybrid(variant) ? 1 : 0;
+  // the passes counts only an instance's group), with the flat passes in
+  // float64
+  b->step = is_hybrid(variant) ? (precision == LSA_FP64 ? 2 : 1) : 0;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(b->w + b->BL.inst, b->inst.data(), (size_t)count * sizeof(BatchInst),
                                   cudaMemcpyHostToDevice, s);
@@ -330,18 +341,18 @@ lsa_status lsa_batch_set_tiling(lsa_batch* b, int group_size, int nlarge) {
 
 lsa_status lsa_batch_set_step_form(lsa_batch* b, int two_phase) {
   if (!b || (two_phase != 0 && two_phase != 1)) return LSA_ERR_ARG;
-  b->two_phase = two_phase;
+  b->step = two_phase;
   return LSA_OK;
 }
 
-int lsa_batch_step_form(const lsa_batch* b) { return b ? b->two_phase : -1; }
+int lsa_batch_step_form(const lsa_batch* b) { return b ? (b->step ? 1 : 0) : -1; }
 
 lsa_status lsa_batch_run(lsa_batch* b, const double* v, double* y, int use_graph, void* stream) {
   if (!b || !v || !y) return LSA_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   if (!use_graph) return b->enqueue(v, y, s) == cudaSuccess ? LSA_OK : LSA_ERR_CUDA;
   if (!(b->gexec && b->gv == v && b->gy == y && b->g_gsize == b->gsize && b->g_nlarge == b->nlarge &&
-        b->g_two == b->two_phase)) {
+        b->g_two == b->step)) {
     b->drop_graph();
     if (!b->cap && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {
       b->cap = nullptr;
@@ -363,7 +374,7 @@ lsa_status lsa_batch_run(lsa_batch* b, const double* v, double* y, int use_graph
     b->gv = v;
     b->gy = y;
     b->g_gsize = b->gsize;
-    b->g_two = b->two_phase;
+    b->g_two = b->step;
     b->g_nlarge = b->nlarge;
   }
   return cudaGraphLaunch(b->gexec, s) == cudaSuccess ? LSA_OK : LSA_ERR_CUDA;
@@ -432,7 +443,7 @@ lsa_status lsa_batch_tune(lsa_batch* b, const double* v, double* y, int reps, in
   auto time_it = [&](int g, int nl, int two) -> float {
     b->gsize = g;
     b->nlarge = nl;
-    b->two_phase = two;
+    b->step = two;
     if (b->enqueue(v, y, s) != cudaSuccess) { result = LSA_ERR_CUDA; return -1.f; }
     float tmin = 1e30f;
     for (int r = 0; r < reps; ++r) {
@@ -449,7 +460,7 @@ lsa_status lsa_batch_tune(lsa_batch* b, const double* v, double* y, int reps, in
     if (st < 0) { result = st; return -1.f; }
     return tmin;
   };
-  const int two0 = b->two_phase;
+  const int two0 = b->step;
   float best = 1e30f;
   Cand bc = {b->gsize, b->nlarge};
   int btwo = two0;
@@ -458,16 +469,18 @@ lsa_status lsa_batch_tune(lsa_batch* b, const double* v, double* y, int reps, in
     if (t < 0.f) break;
     if (t < best) { best = t; bc = c; }
   }
-  // then the other step form of the hybrid variants on the best tiling
-  if (result == LSA_OK && is_hybrid(b->variant)) {
-    const float t = time_it(bc.g, bc.nl, 1 - two0);
-    if (t >= 0.f && t < best) { best = t; btwo = 1 - two0; }
+  // then the other step forms of the hybrid variants on the best tiling
+  const int nforms = b->precision == LSA_FP64 ? 3 : 2;
+  for (int form = 0; form < nforms && result == LSA_OK && is_hybrid(b->variant); ++form) {
+    if (form == two0) continue;
+    const float t = time_it(bc.g, bc.nl, form);
+    if (t >= 0.f && t < best) { best = t; btwo = form; }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   b->gsize = bc.g;
   b->nlarge = bc.nl;
-  b->two_phase = btwo;
+  b->step = btwo;
   if (group_size) *group_size = bc.g;
   if (nlarge) *nlarge = bc.nl;
   if (ms_best) *ms_best = best;

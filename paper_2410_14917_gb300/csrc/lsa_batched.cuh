@@ -12,12 +12,13 @@
 // so the cheap instances fill the tail left by the expensive ones.
 // gsize = grid with nlarge = count is "the whole grid per instance" and
 // nlarge = 0 is "one CTA per instance"; the host-side tuner picks in between,
-// and the step form of the hybrid variants (one-pass or two-phase, whose
-// barrier between its passes is counted over the group).
+// and the step form of the hybrid variants (the flat two-phase passes of
+// lsa_flat.cuh over the group's shares, or the tile passes, one-pass or
+// two-phase; the barrier between two passes is counted over the group).
 #pragma once
 
-#include "lsa_engine.cuh"
 #include "lsa_expm.cuh"
+#include "lsa_flat.cuh"
 
 namespace lsa {
 
@@ -32,6 +33,7 @@ struct BatchInst {      // one instance, with its slice of the workspace
   double* H;            // (m+1) x m
   double* C;            // (PMAX+2) x (MMAX+2) coefficients
   void* V;              // N x (m+3): basis, then the two matvec buffers
+  int2* F;              // limbs of the basis for the flat passes (float64; or null)
 };
 
 struct BatchMail {      // group-queue claim of one group, published by its first CTA
@@ -63,7 +65,7 @@ struct BatchParams {
   const BatchInst* inst;
   const int* order;        // group queue (nlarge entries) then single queue
   int count, nlarge, gsize;
-  int two_phase;           // hybrid variants: the two-phase step (see ArnoldiParams)
+  int step;                // hybrid variants: 0 one-pass, 1 two-phase over tiles, 2 flat two-phase (float64)
   int variant, p;
   double h, tol, brk_tol;
   long long timeout_ns;
@@ -76,15 +78,49 @@ struct BatchParams {
 
 constexpr size_t kMatsPerWorker = (size_t)6 * SMALL_STRIDE * SMALL_STRIDE;
 
+// Barrier of the group after its Arnoldi process: the lead CTA's results (dimension, status, H) are out before
+// any CTA reads them.
+template <class E>
+__device__ __forceinline__ bool batch_results_out(E& e) {
+  e.bt1 += (unsigned)e.gsize;
+  return e.gsize == 1 || e.arrive_wait(&e.P.ctl->arrive, e.bt1, true);
+}
+
+// The Arnoldi process of one instance, with the flat passes or the tile passes.
+template <class Op, class Tc>
+__device__ __noinline__ bool batch_arnoldi_flat(const ArnoldiParams& P, int grank, int gsize, unsigned char* smem) {
+  using F = FlatPass<Op, Tc>;
+  using E = typename F::E;
+  E e(P, *reinterpret_cast<typename E::Smem*>(smem), reinterpret_cast<double*>(smem + E::small_offset()));
+  e.grank = grank;
+  e.gsize = gsize;
+  e.redundant_steps();
+  F f(e, *reinterpret_cast<typename F::Buf*>(smem + F::offset()));
+  f.run();
+  return batch_results_out(e);
+}
+template <class Op, class Tc>
+__device__ __noinline__ bool batch_arnoldi_tiles(const ArnoldiParams& P, int grank, int gsize, unsigned char* smem) {
+  using E = Engine<Op, Tc, Tc>;
+  E e(P, *reinterpret_cast<typename E::Smem*>(smem), reinterpret_cast<double*>(smem + E::small_offset()));
+  e.grank = grank;
+  e.gsize = gsize;
+  e.redundant_steps();
+  e.one_level = true;
+  if (P.variant == LSA_MGS) e.run_mgs(false);
+  else if (P.variant == LSA_CGS2) e.run_cgs2(false);
+  else if (P.variant == LSA_IOCGS) e.run_iocgs(false);
+  else e.run_hybrid();
+  return batch_results_out(e);
+}
+
 // One instance, run by a worker of gsize CTAs (this CTA has rank grank; the
 // worker's scratch index is wbase).  Returns false when a barrier of the
 // instance gave up (the caller leaves the kernel).
 template <class Op, class Tc>
 __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchInst& I, int grank,
                                                int gsize, int wbase,
-                                               typename Engine<Op, Tc, Tc>::Smem& S, double* small,
-                                               ExpmShared& esh, ArnoldiParams& P, SmallParams& SP) {
-  using E = Engine<Op, Tc, Tc>;
+                                               unsigned char* smem, ExpmShared& esh, ArnoldiParams& P, SmallParams& SP) {
   // the parameters live in shared memory (written by one thread): the engine
   // reads them all through, as the standalone kernel reads its parameter bank
   if (threadIdx.x == 0) {
@@ -105,7 +141,8 @@ __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchIn
     P.m = I.m;
     P.variant = BP.variant;
     P.write_vlast = 0;
-    P.two_phase = BP.two_phase;
+    P.two_phase = BP.step;
+    P.F = I.F;
     P.brk_tol = BP.brk_tol;
     P.timeout_ns = BP.timeout_ns;
     SP.H = I.H;
@@ -123,20 +160,13 @@ __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchIn
     SP.tol = BP.tol;
   }
   __syncthreads();
-  {
-    E e(P, S, small);
-    e.grank = grank;
-    e.gsize = gsize;
-    e.redundant_steps();
-    e.one_level = true;
-    if (P.variant == LSA_MGS) e.run_mgs(false);
-    else if (P.variant == LSA_CGS2) e.run_cgs2(false);
-    else if (P.variant == LSA_IOCGS) e.run_iocgs(false);
-    else e.run_hybrid();
-    // the lead CTA's results (dimension, status, H) are out before any CTA of the group reads them
-    e.bt1 += (unsigned)gsize;
-    if (gsize > 1 && !e.arrive_wait(&I.ctl->arrive, e.bt1, true)) return false;
-  }
+  bool ok;
+  if constexpr (sizeof(Tc) == 8)
+    ok = BP.step == 2 && is_hybrid(P.variant) ? batch_arnoldi_flat<Op, Tc>(P, grank, gsize, smem)
+                                              : batch_arnoldi_tiles<Op, Tc>(P, grank, gsize, smem);
+  else
+    ok = batch_arnoldi_tiles<Op, Tc>(P, grank, gsize, smem);
+  if (!ok) return false;
   __syncthreads();
   if (ld_volatile_i32(&I.ctl->abort_flag)) return false;
   if (!expm_group(SP, grank, gsize, esh)) return false;
@@ -162,9 +192,6 @@ __global__ void __launch_bounds__(NT, 2) k_batched(BatchParams BP) {
   __shared__ ArnoldiParams sP;
   __shared__ SmallParams sSP;
   __shared__ int s_idx;
-  using E = Engine<Op, Tc, Tc>;
-  typename E::Smem& S = *reinterpret_cast<typename E::Smem*>(smem_raw);
-  double* small = reinterpret_cast<double*>(smem_raw + E::small_offset());
   const int b = blockIdx.x;
   const int gs = BP.gsize;
   const int ngroups = (BP.nlarge > 0 && gs >= 1) ? (int)gridDim.x / gs : 0;
@@ -205,7 +232,7 @@ __global__ void __launch_bounds__(NT, 2) k_batched(BatchParams BP) {
       if (idx < 0) return;
       if (idx >= BP.nlarge) break;
       const BatchInst& I = BP.inst[BP.order[idx]];
-      if (!batch_instance<Op, Tc>(BP, I, grank, gs, base, S, small, esh, sP, sSP)) {
+      if (!batch_instance<Op, Tc>(BP, I, grank, gs, base, smem_raw, esh, sP, sSP)) {
         if (threadIdx.x == 0) atomicExch(&mb->dead, 1);
         return;
       }
@@ -220,14 +247,20 @@ __global__ void __launch_bounds__(NT, 2) k_batched(BatchParams BP) {
     __syncthreads();
     if (idx >= nsingle) break;
     const BatchInst& I = BP.inst[BP.order[BP.nlarge + idx]];
-    if (!batch_instance<Op, Tc>(BP, I, 0, 1, b, S, small, esh, sP, sSP)) return;
+    if (!batch_instance<Op, Tc>(BP, I, 0, 1, b, smem_raw, esh, sP, sSP)) return;
   }
+}
+
+template <class Op, class Tc>
+constexpr size_t batched_smem_bytes() {
+  const size_t a = Engine<Op, Tc, Tc>::smem_bytes(), b = sizeof(Tc) == 8 ? FlatPass<Op, Tc>::smem_bytes() : 0;
+  return a > b ? a : b;
 }
 
 template <class Op, class Tc>
 cudaError_t launch_batched_t(const BatchParams& BP, int G, cudaStream_t s) {
   auto k = k_batched<Op, Tc>;
-  const size_t sm = Engine<Op, Tc, Tc>::smem_bytes();
+  const size_t sm = batched_smem_bytes<Op, Tc>();
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   // cooperative launch (all CTAs co-resident: the group barriers and the
@@ -257,12 +290,12 @@ int batched_blocks_per_sm_op(int precision) {
   int nb = 0;
   if (precision == LSA_FP64) {
     auto k = k_batched<Op, double>;
-    const size_t sm = Engine<Op, double, double>::smem_bytes();
+    const size_t sm = batched_smem_bytes<Op, double>();
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, sm);
   } else {
     auto k = k_batched<Op, float>;
-    const size_t sm = Engine<Op, float, float>::smem_bytes();
+    const size_t sm = batched_smem_bytes<Op, float>();
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, sm);
   }
