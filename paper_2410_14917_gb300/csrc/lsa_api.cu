@@ -14,9 +14,9 @@ namespace lsa {
 cudaError_t launch_arnoldi_advdiff2d(const ArnoldiParams&, int, int, cudaStream_t);
 cudaError_t launch_arnoldi_grayscott2d(const ArnoldiParams&, int, int, cudaStream_t);
 cudaError_t launch_arnoldi_adr3d(const ArnoldiParams&, int, int, cudaStream_t);
-cudaError_t launch_matvec_advdiff2d(const ArnoldiParams&, int, const void*, void*, int, cudaStream_t);
-cudaError_t launch_matvec_grayscott2d(const ArnoldiParams&, int, const void*, void*, int, cudaStream_t);
-cudaError_t launch_matvec_adr3d(const ArnoldiParams&, int, const void*, void*, int, cudaStream_t);
+cudaError_t launch_matvec_advdiff2d(const ArnoldiParams&, int, const void*, void*, cudaStream_t);
+cudaError_t launch_matvec_grayscott2d(const ArnoldiParams&, int, const void*, void*, cudaStream_t);
+cudaError_t launch_matvec_adr3d(const ArnoldiParams&, int, const void*, void*, cudaStream_t);
 int blocks_per_sm_advdiff2d(int);
 int blocks_per_sm_grayscott2d(int);
 int blocks_per_sm_adr3d(int);
@@ -44,10 +44,10 @@ cudaError_t launch_arnoldi_cluster_advdiff2d(const ArnoldiParams&, const SmallPa
 cudaError_t launch_arnoldi_stream_adr3d(const ArnoldiParams&, cudaStream_t);
 
 cudaError_t launch_arnoldi_grayscott2d_t(const ArnoldiParams&, int, int, cudaStream_t);
-cudaError_t launch_matvec_grayscott2d_t(const ArnoldiParams&, int, const void*, void*, int, cudaStream_t);
+cudaError_t launch_matvec_grayscott2d_t(const ArnoldiParams&, int, const void*, void*, cudaStream_t);
 int blocks_per_sm_grayscott2d_t(int);
 cudaError_t launch_arnoldi_grayscott2d_frechet(const ArnoldiParams&, int, int, cudaStream_t);
-cudaError_t launch_matvec_grayscott2d_frechet(const ArnoldiParams&, int, const void*, void*, int, cudaStream_t);
+cudaError_t launch_matvec_grayscott2d_frechet(const ArnoldiParams&, int, const void*, void*, cudaStream_t);
 int blocks_per_sm_grayscott2d_frechet(int);
 
 static const long long kTimeoutNs = 5000000000LL;   // 5 s per barrier wait
@@ -365,14 +365,13 @@ static cudaError_t launch_arnoldi_grid(const ArnoldiParams& P, int precision, in
   return launch_arnoldi_adr3d(P, precision, G, s);
 }
 
-cudaError_t launch_matvec(const ArnoldiParams& P, int precision, const void* x, void* y, int G,
-                          cudaStream_t s) {
-  if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_matvec_advdiff2d(P, precision, x, y, G, s);
-  if (P.op.kind == LSA_OP_GRAYSCOTT2D) return launch_matvec_grayscott2d(P, precision, x, y, G, s);
-  if (P.op.kind == LSA_OP_GRAYSCOTT2D_T) return launch_matvec_grayscott2d_t(P, precision, x, y, G, s);
+cudaError_t launch_matvec(const ArnoldiParams& P, int precision, const void* x, void* y, cudaStream_t s) {
+  if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_matvec_advdiff2d(P, precision, x, y, s);
+  if (P.op.kind == LSA_OP_GRAYSCOTT2D) return launch_matvec_grayscott2d(P, precision, x, y, s);
+  if (P.op.kind == LSA_OP_GRAYSCOTT2D_T) return launch_matvec_grayscott2d_t(P, precision, x, y, s);
   if (P.op.kind == LSA_OP_GRAYSCOTT2D_FRECHET)
-    return launch_matvec_grayscott2d_frechet(P, precision, x, y, G, s);
-  return launch_matvec_adr3d(P, precision, x, y, G, s);
+    return launch_matvec_grayscott2d_frechet(P, precision, x, y, s);
+  return launch_matvec_adr3d(P, precision, x, y, s);
 }
 
 // Workspace layout for (op, m, precision).  G = CTAs of the persistent kernel.
@@ -569,10 +568,7 @@ lsa_status lsa_matvec(const lsa_op* op, const void* x, void* y, int precision, v
   lsa_status st = prepare(op, 1, precision, work, work_bytes, &pr);
   if (st != LSA_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = launch_init(pr.P.ctl, pr.d, (float*)pr.d.g0, (float*)pr.d.g1, precision, nullptr, 0,
-                              nullptr, nullptr, s);
-  if (e == cudaSuccess) e = launch_matvec(pr.P, precision, x, y, pr.L.G, s);
-  return from_cuda(e);
+  return from_cuda(launch_matvec(pr.P, precision, x, y, s));
 }
 
 lsa_status lsa_arnoldi(const lsa_op* op, const double* v, int m, int variant, int precision,

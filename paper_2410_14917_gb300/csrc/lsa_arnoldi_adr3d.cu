@@ -9,8 +9,8 @@ cudaError_t launch_arnoldi_adr3d(const ArnoldiParams& P, int precision, int G, c
   return launch_arnoldi_op<OpADR3D>(P, precision, G, s);
 }
 cudaError_t launch_matvec_adr3d(const ArnoldiParams& P, int precision, const void* x, void* y,
-                                int G, cudaStream_t s) {
-  return launch_matvec_op<OpADR3D>(P, precision, x, y, G, s);
+                                        cudaStream_t s) {
+  return launch_matvec_op<OpADR3D>(P, precision, x, y, s);
 }
 int blocks_per_sm_adr3d(int precision) { return blocks_per_sm_op<OpADR3D>(precision); }
 bool tma_applicable_adr3d(const DevOp& d, const Tiling& tl, int m, int precision) {

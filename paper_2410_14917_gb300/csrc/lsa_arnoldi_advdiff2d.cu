@@ -10,8 +10,8 @@ cudaError_t launch_arnoldi_advdiff2d(const ArnoldiParams& P, int precision, int 
   return launch_arnoldi_op<OpAdvDiff2D>(P, precision, G, s);
 }
 cudaError_t launch_matvec_advdiff2d(const ArnoldiParams& P, int precision, const void* x, void* y,
-                                int G, cudaStream_t s) {
-  return launch_matvec_op<OpAdvDiff2D>(P, precision, x, y, G, s);
+                                        cudaStream_t s) {
+  return launch_matvec_op<OpAdvDiff2D>(P, precision, x, y, s);
 }
 int blocks_per_sm_advdiff2d(int precision) { return blocks_per_sm_op<OpAdvDiff2D>(precision); }
 bool tma_applicable_advdiff2d(const DevOp& d, const Tiling& tl, int m, int precision) {

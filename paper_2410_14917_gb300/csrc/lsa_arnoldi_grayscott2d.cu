@@ -8,8 +8,8 @@ cudaError_t launch_arnoldi_grayscott2d(const ArnoldiParams& P, int precision, in
   return launch_arnoldi_op<OpGrayScott2D>(P, precision, G, s);
 }
 cudaError_t launch_matvec_grayscott2d(const ArnoldiParams& P, int precision, const void* x, void* y,
-                                int G, cudaStream_t s) {
-  return launch_matvec_op<OpGrayScott2D>(P, precision, x, y, G, s);
+                                        cudaStream_t s) {
+  return launch_matvec_op<OpGrayScott2D>(P, precision, x, y, s);
 }
 int blocks_per_sm_grayscott2d(int precision) { return blocks_per_sm_op<OpGrayScott2D>(precision); }
 bool tma_applicable_grayscott2d(const DevOp& d, const Tiling& tl, int m, int precision) {

@@ -1643,19 +1643,43 @@ __global__ void __launch_bounds__(NT, (sizeof(Tc) == 8) ? LSA_MINB_F64 : LSA_MIN
   else e.run_hybrid();
 }
 
-// One stencil pass y = A x with the same tile code (no barrier).
-template <class Op, class Tc, class B>
-__global__ void __launch_bounds__(NT) k_matvec(ArnoldiParams P, const B* x, B* y) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using E = Engine<Op, Tc, B>;
-  typename E::Smem& S = *reinterpret_cast<typename E::Smem*>(smem_raw);
-  E e(P, S, reinterpret_cast<double*>(smem_raw + E::small_offset()));
-  if (threadIdx.x == 0) S.a = (Tc)1;
-  __syncthreads();
-  PassT<B> ps;
-  ps.c0 = ps.c1 = 0; ps.a = 1.0; ps.src64 = nullptr; ps.srcB = x;
-  ps.xout = nullptr; ps.wout = y; ps.d0 = ps.d1 = 0; ps.dmode = 0; ps.self = 0;
-  e.run_pass(ps);
+// y = A x, one thread per grid point (all its species), neighbours through L1; the operator's own arithmetic,
+// so y is bitwise the Arnoldi passes' value.  The float32 form makes its copies of the fields on the fly, so one
+// launch does (it was two, the second over persistent CTAs with barriers per tile: 22 us a call on Gray-Scott
+// 512^2, 14.3 us now, launch included).
+template <class Op, class Tc>
+__global__ void __launch_bounds__(NT) k_matvec(DevOp d, Coef<Tc> cf, const Tc* __restrict__ x, Tc* __restrict__ y,
+                                              Ctl* ctl) {
+  constexpr int NS = Op::NS;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < (int)(sizeof(Ctl) / sizeof(int)); i += NT) reinterpret_cast<int*>(ctl)[i] = 0;
+  const long long g = blockIdx.x * (long long)NT + threadIdx.x;
+  if (g >= d.npts) return;
+  const int q = (int)g, nxy = d.nx * d.ny;
+  const int r = q / d.nx, ix = q - r * d.nx;
+  const int iz = r / d.ny, iy = r - iz * d.ny;
+  const int qw = ix == 0 ? q + (d.nx - 1) : q - 1, qe = ix == d.nx - 1 ? q - (d.nx - 1) : q + 1;
+  const int qs = iy == 0 ? q + (d.ny - 1) * d.nx : q - d.nx, qn = iy == d.ny - 1 ? q - (d.ny - 1) * d.nx : q + d.nx;
+  Tc c5[5 * NS], zm[3], zp[3], out[NS], f0 = (Tc)0, f1 = (Tc)0;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const Tc* xs = x + s * d.npts;
+    c5[5 * s] = xs[qs]; c5[5 * s + 1] = xs[qw]; c5[5 * s + 2] = xs[q]; c5[5 * s + 3] = xs[qe]; c5[5 * s + 4] = xs[qn];
+  }
+  zm[0] = zm[1] = zm[2] = zp[0] = zp[1] = zp[2] = (Tc)0;
+  if constexpr (Op::DIM == 3) {
+    zm[2] = x[iz == 0 ? q + (d.nz - 1) * nxy : q - nxy];
+    zp[2] = x[iz == d.nz - 1 ? q - (d.nz - 1) * nxy : q + nxy];
+  }
+  if constexpr (Op::NF == 1) f0 = (Tc)__ldg(d.f0 + q);
+  if constexpr (Op::NF == 2) {
+    const double u0 = __ldg(d.f0 + q), v0 = __ldg(d.f1 + q);
+    f0 = sizeof(Tc) == 8 ? (Tc)u0 : (Tc)(v0 * v0);
+    f1 = sizeof(Tc) == 8 ? (Tc)v0 : (Tc)(2.0 * u0 * v0);
+  }
+  Op::template apply_f<Tc, 2, 5>(cf, zm, c5, zp, 2, f0, f1, out);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) y[s * d.npts + q] = out[s];
 }
 
 template <class Op, class Tc>
@@ -1676,12 +1700,11 @@ cudaError_t launch_arnoldi_t(const ArnoldiParams& P, int G, cudaStream_t s) {
 }
 
 template <class Op, class Tc>
-cudaError_t launch_matvec_t(const ArnoldiParams& P, const void* x, void* y, int G, cudaStream_t s) {
-  auto k = k_matvec<Op, Tc, Tc>;
-  size_t sm = Engine<Op, Tc, Tc>::smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  k<<<G, NT, sm, s>>>(P, (const Tc*)x, (Tc*)y);
+cudaError_t launch_matvec_t(const ArnoldiParams& P, const void* x, void* y, cudaStream_t s) {
+  const long long blocks = (P.op.npts + NT - 1) / NT;
+  Coef<Tc> cf;
+  cf.load(P.op);
+  k_matvec<Op, Tc><<<(unsigned)blocks, NT, 0, s>>>(P.op, cf, (const Tc*)x, (Tc*)y, P.ctl);
   return cudaGetLastError();
 }
 
@@ -1701,10 +1724,8 @@ cudaError_t launch_arnoldi_op(const ArnoldiParams& P, int precision, int G, cuda
 }
 
 template <class Op>
-cudaError_t launch_matvec_op(const ArnoldiParams& P, int precision, const void* x, void* y, int G,
-                             cudaStream_t s) {
-  return precision == LSA_FP64 ? launch_matvec_t<Op, double>(P, x, y, G, s)
-                               : launch_matvec_t<Op, float>(P, x, y, G, s);
+cudaError_t launch_matvec_op(const ArnoldiParams& P, int precision, const void* x, void* y, cudaStream_t s) {
+  return precision == LSA_FP64 ? launch_matvec_t<Op, double>(P, x, y, s) : launch_matvec_t<Op, float>(P, x, y, s);
 }
 
 template <class Op>

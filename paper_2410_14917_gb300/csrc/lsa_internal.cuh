@@ -152,8 +152,7 @@ size_t workspace_least_bytes(const lsa_op* op, int m, int p, int precision);
 
 // Launchers implemented per operator translation unit.
 cudaError_t launch_arnoldi(const ArnoldiParams& P, int precision, int G, cudaStream_t s);
-cudaError_t launch_matvec(const ArnoldiParams& P, int precision, const void* x, void* y, int G,
-                          cudaStream_t s);
+cudaError_t launch_matvec(const ArnoldiParams& P, int precision, const void* x, void* y, cudaStream_t s);
 int arnoldi_blocks_per_sm(const DevOp& d, int precision);
 
 // Small kernels (lsa_small.cu)

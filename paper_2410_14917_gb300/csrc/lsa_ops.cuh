@@ -15,7 +15,7 @@ template <class Tc>
 struct Coef {
   Tc cW, cE, cS, cN, cD, cU, cC, du, dv, F, k, idx2;
   int dir;
-  __device__ void load(const DevOp& d) {
+  __host__ __device__ void load(const DevOp& d) {
     cW = (Tc)d.cW; cE = (Tc)d.cE; cS = (Tc)d.cS; cN = (Tc)d.cN;
     cD = (Tc)d.cD; cU = (Tc)d.cU; cC = (Tc)d.cC;
     du = (Tc)d.du; dv = (Tc)d.dv; F = (Tc)d.F; k = (Tc)d.k; idx2 = (Tc)d.idx2;
