@@ -19,9 +19,13 @@ namespace lsa {
 // The polynomial is evaluated by the Paterson-Stockmeyer scheme with blocks of
 // four powers (X^2, X^3, X^4, then four Horner steps in X^4), so the whole
 // exponential is 7 + s matrix products with no linear solve.  Every product is
-// spread over all CTAs of a cooperative launch (one output entry per thread),
-// because FP64 arithmetic on this part is ~64x slower than FP32 and a single
-// SM would take hundreds of microseconds.
+// spread over all CTAs of a cooperative launch, because FP64 arithmetic on this
+// part is ~64x slower than FP32 and a single SM would take hundreds of
+// microseconds.  A product's time is its round trips to L2 and the barrier
+// after it, so up to four threads share an entry (few, long batches of loads)
+// and the barrier is one counter that every CTA polls: 18 to 20 us less a call
+// at n = 26 and n = 34 (advection-diffusion 64 x 64 with m = 30: 424 to 405 us)
+// than with one thread per entry and a release flag.
 
 constexpr int EXPM_NT = 64;
 constexpr int LD = SMALL_STRIDE;
@@ -31,7 +35,7 @@ struct ExpmShared {
   int flag;
   int m, n, s;
   double scale;
-  double nrm[NT];
+  double nrm[NT / 32];
 };
 
 __device__ __forceinline__ double hhat(const SmallParams& P, int m, double scale, int r, int c) {
@@ -42,28 +46,28 @@ __device__ __forceinline__ double hhat(const SmallParams& P, int m, double scale
   return v * scale;
 }
 
-// sum_k A[r][k] B[k][c] over k < n (leading dimension LD): eight loads of each
-// operand in flight per round trip to L2 (a product entry is one thread's
-// chain, so its loads, not its FMAs, set the time), four accumulators
-// combined in a fixed order.
-__device__ __forceinline__ double dot_rc(const double* A, const double* B, int r, int c, int n) {
+// This thread's share of sum_k A[r][k] B[k][c], k = q, q + S, ... < n (leading dimension LD): up to eight
+// loads of each operand in flight per round trip to L2, two accumulators.
+__device__ __forceinline__ double dot_rc(const double* A, const double* B, int r, int c, int n, int q, int S) {
   const double* a = A + r * LD;
   const double* b = B + c;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  for (int k = 0; k < n; k += 8) {
+  double s0 = 0.0, s1 = 0.0;
+  for (int k = q; k < n; k += 8 * S) {
     double x[8], y[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const bool in = k + i < n;
-      x[i] = in ? __ldcg(a + k + i) : 0.0;
-      y[i] = in ? __ldcg(b + (k + i) * LD) : 0.0;
+      const int kk = k + i * S;
+      const bool in = kk < n;
+      x[i] = in ? __ldcg(a + kk) : 0.0;
+      y[i] = in ? __ldcg(b + kk * LD) : 0.0;
     }
-    s0 = fma(x[0], y[0], s0); s1 = fma(x[1], y[1], s1);
-    s2 = fma(x[2], y[2], s2); s3 = fma(x[3], y[3], s3);
-    s0 = fma(x[4], y[4], s0); s1 = fma(x[5], y[5], s1);
-    s2 = fma(x[6], y[6], s2); s3 = fma(x[7], y[7], s3);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      s0 = fma(x[i], y[i], s0);
+      s1 = fma(x[i + 1], y[i + 1], s1);
+    }
   }
-  return (s0 + s1) + (s2 + s3);
+  return s0 + s1;
 }
 
 // B_l = sum_{i=0}^{3} a_{4l+i} X^i  (a_k = 1/k!; B_4 = a16 I + a17 X + a18 X^2)
@@ -110,38 +114,45 @@ static __device__ __noinline__ bool expm_group(const SmallParams& P, int grank, 
   double* R0 = X4 + LD * LD;
   double* R1 = R0 + LD * LD;
 
-  // the closing group barrier of the early exits (generation 0: no product ran)
-  auto close0 = [&]() -> bool {
+  // group barrier: the CTAs' arrivals at one counter, which all of them poll
+  unsigned target = 0;
+  auto barrier = [&]() -> bool {
     if constexpr (kCluster) {
       __syncthreads();
       cluster_barrier();
       return true;
     }
-    int r = barrier_arrive(br, 0u, G, &sh.flag, P.timeout_ns);
-    if (r < 0) return false;
-    if (r == 1) barrier_release(br, 0u);
-    return true;
+    target += G;
+    return counter_barrier(br, target, &sh.flag, P.timeout_ns);
   };
 
   if (m == 0) {   // zero start vector or failed Arnoldi: all coefficients zero
     for (int i = grank * nthr + tid; i < (p + 2) * P.ldc; i += G * nthr) P.C[i] = 0.0;
     if (grank == 0 && tid == 0) ctl->err_est = 0.0;
-    return close0();
+    return barrier();
   }
 
-  // ||Hhat||_1 = max(1, max_c sum_r |h H_rc|), computed redundantly by every CTA
+  // ||Hhat||_1 = max(1, max_c sum_r |h H_rc|), computed redundantly by every CTA: sixteen loads in flight
   {
     double mx = 0.0;
     for (int c = tid; c < m; c += nthr) {
-      double s = 0.0;
-      for (int r = 0; r < m; ++r) s += fabs(P.h * __ldcg(P.H + r + (long long)c * P.ldh));
-      mx = fmax(mx, s);
+      double t = 0.0;
+      for (int r = 0; r < m; r += 16) {
+        double v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = r + i < m ? __ldcg(P.H + r + i + (long long)c * P.ldh) : 0.0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) t += fabs(P.h * v[i]);
+      }
+      mx = fmax(mx, t);
     }
-    sh.nrm[tid] = mx;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) sh.nrm[tid >> 5] = mx;
     __syncthreads();
     if (tid == 0) {
       double v = 1.0;
-      for (int i = 0; i < nthr; ++i) v = fmax(v, sh.nrm[i]);
+      for (int i = 0; i < nthr / 32; ++i) v = fmax(v, sh.nrm[i]);
       int s = 0;
       if (!isfinite(v)) s = -1;
       else while (v > 1.0 && s < 1000) { v *= 0.5; ++s; }
@@ -155,26 +166,30 @@ static __device__ __noinline__ bool expm_group(const SmallParams& P, int grank, 
       atomicCAS(&ctl->status, 0, (int)LSA_ERR_NUMERIC);
       ctl->err_est = 0.0;
     }
-    return close0();
+    return barrier();
   }
   const int s = sh.s;
   const double scale = sh.scale;
-  unsigned gen = 0;
   const int gtid = grank * nthr + tid;
   const int gstride = G * nthr;
   const int nn = n * n;
+  // f(o, q, S) for the entries o < total: S threads of a warp share an entry and add up their values
+  auto entries = [&](int total, auto f, auto store) {
+    int S = 4;
+    while (S > 1 && (long long)total * S > gstride) S >>= 1;
+    const int rounds = (total * S + gstride - 1) / gstride, q = gtid % S;
+    for (int i = 0; i < rounds; ++i) {
+      const int o = (gtid + i * gstride) / S;
+      double v = o < total ? f(o, q, S) : 0.0;
+      if (S > 1) v += __shfl_xor_sync(0xffffffffu, v, 1);
+      if (S > 2) v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (q == 0 && o < total) store(o, v);
+    }
+  };
 
-#define EXPM_BARRIER()                                                          \
-  do {                                                                          \
-    if constexpr (kCluster) {                                                   \
-      __syncthreads();                                                          \
-      cluster_barrier();                                                        \
-    } else {                                                                    \
-      int _r = barrier_arrive(br, gen, G, &sh.flag, P.timeout_ns);              \
-      if (_r < 0) return false;                                                 \
-      if (_r == 1) barrier_release(br, gen);                                    \
-    }                                                                           \
-    ++gen;                                                                      \
+#define EXPM_BARRIER()              \
+  do {                              \
+    if (!barrier()) return false;   \
   } while (0)
 
   // X = Hhat * 2^-s
@@ -184,56 +199,57 @@ static __device__ __noinline__ bool expm_group(const SmallParams& P, int grank, 
   }
   EXPM_BARRIER();
   // X2 = X X
-  for (int o = gtid; o < nn; o += gstride) {
-    int r = o / n, c = o - r * n;
-    X2[r * LD + c] = dot_rc(X, X, r, c, n);
-  }
+  entries(nn, [&](int o, int q, int S) { return dot_rc(X, X, o / n, o % n, n, q, S); },
+          [&](int o, double v) { X2[(o / n) * LD + o % n] = v; });
   EXPM_BARRIER();
   // X3 = X2 X, X4 = X2 X2
-  for (int o = gtid; o < 2 * nn; o += gstride) {
-    int which = o >= nn;
-    int oo = o - which * nn;
-    int r = oo / n, c = oo - r * n;
-    (which ? X4 : X3)[r * LD + c] = dot_rc(X2, which ? X2 : X, r, c, n);
-  }
+  entries(2 * nn,
+          [&](int o, int q, int S) {
+            const int which = o >= nn, oo = o - which * nn;
+            return dot_rc(X2, which ? X2 : X, oo / n, oo % n, n, q, S);
+          },
+          [&](int o, double v) {
+            const int which = o >= nn, oo = o - which * nn;
+            (which ? X4 : X3)[(oo / n) * LD + oo % n] = v;
+          });
   EXPM_BARRIER();
   // Horner in X^4: R = B_4; R = B_l + X^4 R for l = 3, 2, 1, 0
   double* Rin = R0;
   double* Rout = R1;
   for (int l = 3; l >= 0; --l) {
-    for (int o = gtid; o < nn; o += gstride) {
-      int r = o / n, c = o - r * n;
-      double acc;
-      if (l < 3) {
-        acc = dot_rc(X4, Rin, r, c, n);
-      } else {                           // R = B_4 formed on the fly: eight of its entries per round trip
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        for (int k = 0; k < n; k += 8) {
-          double x[8], y[8];
+    entries(nn,
+            [&](int o, int q, int S) {
+              const int r = o / n, c = o % n;
+              if (l < 3) return dot_rc(X4, Rin, r, c, n, q, S);
+              double s0 = 0.0, s1 = 0.0;        // R = B_4 formed on the fly
+              for (int k = q; k < n; k += 8 * S) {
+                double x[8], y[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const bool in = k + i < n;
-            x[i] = in ? __ldcg(X4 + r * LD + k + i) : 0.0;
-            y[i] = in ? block_coef(X, X2, X3, 4, k + i, c, a) : 0.0;
-          }
-          s0 = fma(x[0], y[0], s0); s1 = fma(x[1], y[1], s1);
-          s2 = fma(x[2], y[2], s2); s3 = fma(x[3], y[3], s3);
-          s0 = fma(x[4], y[4], s0); s1 = fma(x[5], y[5], s1);
-          s2 = fma(x[6], y[6], s2); s3 = fma(x[7], y[7], s3);
-        }
-        acc = (s0 + s1) + (s2 + s3);
-      }
-      Rout[r * LD + c] = block_coef(X, X2, X3, l, r, c, a) + acc;
-    }
+                for (int i = 0; i < 8; ++i) {
+                  const int kk = k + i * S;
+                  const bool in = kk < n;
+                  x[i] = in ? __ldcg(X4 + r * LD + kk) : 0.0;
+                  y[i] = in ? block_coef(X, X2, X3, 4, kk, c, a) : 0.0;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) {
+                  s0 = fma(x[i], y[i], s0);
+                  s1 = fma(x[i + 1], y[i + 1], s1);
+                }
+              }
+              return s0 + s1;
+            },
+            [&](int o, double v) {
+              const int r = o / n, c = o % n;
+              Rout[r * LD + c] = block_coef(X, X2, X3, l, r, c, a) + v;
+            });
     EXPM_BARRIER();
     double* t = Rin; Rin = Rout; Rout = t;
   }
   // squarings
-  for (int q = 0; q < s; ++q) {
-    for (int o = gtid; o < nn; o += gstride) {
-      int r = o / n, c = o - r * n;
-      Rout[r * LD + c] = dot_rc(Rin, Rin, r, c, n);
-    }
+  for (int q2 = 0; q2 < s; ++q2) {
+    entries(nn, [&](int o, int q, int S) { return dot_rc(Rin, Rin, o / n, o % n, n, q, S); },
+            [&](int o, double v) { Rout[(o / n) * LD + o % n] = v; });
     EXPM_BARRIER();
     double* t = Rin; Rin = Rout; Rout = t;
   }

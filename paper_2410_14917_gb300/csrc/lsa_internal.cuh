@@ -345,6 +345,35 @@ __device__ __forceinline__ int counter_arrive(unsigned* ctr, unsigned gen, unsig
   return *s_flag;
 }
 
+// Group barrier on one counter: every CTA adds its arrival and polls until `target` have been counted (bounded
+// like barrier_arrive; false on a timeout or abort).
+__device__ __forceinline__ bool counter_barrier(const BarrierRef& b, unsigned target, int* s_flag, long long timeout_ns) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(b.arrive, 1u);
+    int ok = 1;
+    unsigned it = 0;
+    const unsigned long long t0 = global_ns();
+    while ((int)(ld_acquire_u32(b.arrive) - target) < 0) {
+      if ((++it & 255u) == 0u) {
+        if (ld_volatile_i32(b.abort_flag)) { ok = 0; break; }
+        if ((long long)(global_ns() - t0) > timeout_ns) {
+          atomicExch(b.abort_flag, 1);
+          atomicCAS(b.status, 0, (int)LSA_ERR_TIMEOUT);
+          ok = 0;
+          break;
+        }
+        if (it > 4096u) __nanosleep(64);
+      }
+    }
+    __threadfence();
+    *s_flag = ok;
+  }
+  __syncthreads();
+  return *s_flag != 0;
+}
+
 __device__ __forceinline__ void barrier_release(const BarrierRef& b, unsigned gen) {
   __syncthreads();
   if (threadIdx.x == 0) {
