@@ -21,6 +21,10 @@
 //    memory) and stores the next pass's coefficients and flags straight into
 //    every CTA's shared memory; a second cluster barrier releases the others.
 //
+//  * the pass's inner products, two FMAs per column value and bound by the
+//    float64 unit of its 16 SMs, are exact integer sums instead (lsa_fix.cuh):
+//    64 x 64 with m = 30 takes 344 us a phi product, 405 with float64 products.
+//
 // Per Alg. 4 step: three cluster barriers (halo ready, partials ready, step
 // published) and no global-memory barrier.  The hardware cluster barrier has
 // no timeout to bound: every CTA follows the same control flow (its decisions
@@ -29,6 +33,7 @@
 
 #include "lsa_engine.cuh"
 #include "lsa_expm.cuh"
+#include "lsa_fix.cuh"
 
 namespace lsa {
 
@@ -67,6 +72,14 @@ __device__ __forceinline__ void cl_st(int* local, unsigned rank, int v) {
 // of the O(j^2) step, which holds T, and GSMGS's L, between steps in CTA 0):
 // the tile's basis [m+3][CL_TP] (columns 0..m, then the two
 // matvec buffers m+1, m+2) and the CTA's partial sums [SLOTS].
+// The tile's x and w as limbs (xh, xl, wh, wl), and the largest keys of its slice of every column and of w
+// (lsa_fix.cuh).
+struct ClusterFix {
+  int4 xw[CL_TP];
+  unsigned ckey[MMAX + 2];
+  unsigned wkey;
+};
+
 template <class Op>
 struct ClusterLayout {
   using E = Engine<Op, double, double>;
@@ -80,9 +93,10 @@ struct ClusterLayout {
   static __host__ __device__ constexpr size_t cs_off(int m) {
     return (expm_off(m) + sizeof(ExpmShared) + 15) & ~(size_t)15;
   }
-  static __host__ __device__ constexpr size_t bytes(int m) {
-    return cs_off(m) + sizeof(double) * (PMAX + 1) * (MMAX + 2);
+  static __host__ __device__ constexpr size_t fix_off(int m) {
+    return (cs_off(m) + sizeof(double) * (PMAX + 1) * (MMAX + 2) + 15) & ~(size_t)15;
   }
+  static __host__ __device__ constexpr size_t bytes(int m) { return fix_off(m) + sizeof(ClusterFix); }
 };
 
 template <class Op>
@@ -93,10 +107,11 @@ struct ClusterEngine {
   E& e;
   double* Vt;      // this tile's basis slice
   double* part;    // this CTA's partial sums
+  ClusterFix& fx;
   const int lx, ly, gx, gy, gi;
 
-  __device__ ClusterEngine(E& en, double* vt, double* pt)
-      : e(en), Vt(vt), part(pt), lx(en.tid & (TX - 1)), ly(en.tid / TX),
+  __device__ ClusterEngine(E& en, double* vt, double* pt, ClusterFix& f)
+      : e(en), Vt(vt), part(pt), fx(f), lx(en.tid & (TX - 1)), ly(en.tid / TX),
         gx((en.grank % en.P.tl.tiles_x) * TX + (en.tid & (TX - 1))),
         gy((en.grank / en.P.tl.tiles_x) * TY + en.tid / TX),
         gi(gx + en.P.op.nx * gy) {}
@@ -115,10 +130,10 @@ struct ClusterEngine {
   // One pass of the hybrid process over this tile: x = a*src - sum_{c < ncp}
   // coef_c V_c (src < 0: the start vector), stored in column xout (>= 0); with
   // wout >= 0 the stencil w = A x into column wout and the inner products of
-  // columns 0..ncp-1 with x and w; the self terms selected by `self`.  Partial
-  // sums as the grid kernel lays them out (x dots, w dots, then x.x, x.w,
-  // w.w); returns their number.
-  __device__ int pass(int ncp, int src, double a, int xout, int wout, int self) {
+  // columns 0..ncp-1 with x and w, x.x, x.w and w.w; without, x.x.  Partial sums
+  // as the grid kernel lays them out (x dots, w dots, then x.x, x.w, w.w);
+  // returns their number.
+  __device__ int pass(int ncp, int src, double a, int xout, int wout) {
     const int t = e.tid;
     double x = (src < 0) ? a * __ldg(e.P.vin + gi) : a * Vt[(size_t)src * CL_TP + t];
     double xb = 0.0;   // odd columns in a second chain (half the dependency depth)
@@ -129,13 +144,15 @@ struct ClusterEngine {
       else x = fma(-cc, v, x);
     }
     x += xb;
+    const bool stencil = wout >= 0;
     if (xout >= 0) {
       Vt[(size_t)xout * CL_TP + t] = x;
       reinterpret_cast<double*>(e.P.V)[(long long)xout * e.P.op.N + gi] = x;   // write-through
     }
     double w = 0.0;
-    const bool stencil = wout >= 0;
     if (stencil) {
+      const unsigned kx = __reduce_max_sync(0xffffffffu, fx_key(x));
+      if (e.lane == 0) atomicMax(&fx.ckey[xout], kx);     // (zeroed by run_hybrid)
       cl_sync();   // every tile's x is in its CTA's shared memory
       const Coef<double>& cf = e.cf;
       double r = cf.cC * x;
@@ -145,63 +162,74 @@ struct ClusterEngine {
       r = fma(cf.cN, (ly < TY - 1) ? Vt[(size_t)xout * CL_TP + t + TX] : xat(xout, gx, gy + 1), r);
       w = r;
       Vt[(size_t)wout * CL_TP + t] = w;
+      const unsigned kw = __reduce_max_sync(0xffffffffu, fx_key(w));
+      if (e.lane == 0) atomicMax(&fx.wkey, kw);
     }
-    // self terms: block sums
-    double s3[4] = {(self & SELF_XX) ? x * x : 0.0, (self & SELF_XW) ? x * w : 0.0,
-                    (self & SELF_WW) ? w * w : 0.0, 0.0};
+    // self term in float64 (the others are inner products with column xout): warp sums
     {
-      const double r = warp_sum_many<4>(s3);   // lane l: value l >> 3
-      if ((e.lane & 7) == 0 && e.lane < 24) e.S.bred[e.warp][e.lane >> 3] = r;
+      const double r = warp_sum(stencil ? w * w : x * x);
+      if (e.lane == 0) e.S.bred[e.warp][0] = r;
     }
-    __syncthreads();   // x, w and the warp sums are in shared memory
+    __syncthreads();   // x, w, their keys and the warp sums are in shared memory
     const int nd = stencil ? ncp : 0;
-    // inner products: warp <-> columns c = warp, warp + NW, ...; lane <-> points
-    const double* xc = Vt + (size_t)xout * CL_TP;
-    const double* wc = Vt + (size_t)wout * CL_TP;
-    if (nd <= NW) {              // at most one column per warp
-      const int c = e.warp;
-      if (c < nd) {
-        const double* vc = Vt + (size_t)c * CL_TP;
-        double ax = 0.0, aw = 0.0;
+    if (stencil) {
+      const unsigned kw = fx.wkey;
+      int4 q;
+      fx_split0(x, fx_base(fx.ckey[xout]), q.x, q.y);
+      fx_split0(w, fx_base(kw), q.z, q.w);
+      fx.xw[t] = q;
+      __syncthreads();
+      if (t == 0) fx.wkey = 0;
+      // inner products on the integer unit (lsa_fix.cuh): warp <-> columns c = warp, warp + NW, ... <= nd (the
+      // last one is x), lane <-> points
+      auto dot = [&](int c, long long& tx, long long& tw) {
+        const double* vc = Vt + (size_t)c * CL_TP + e.lane;
+        const int4* pt = fx.xw + e.lane;
+        const unsigned base = fx_base(fx.ckey[c]);
+        long long xx = 0, xc = 1LL << 31, ww = 0, wc = 1LL << 31;
 #pragma unroll
         for (int k = 0; k < CL_TP / 32; ++k) {
-          const int q = e.lane + 32 * k;
-          ax = fma(vc[q], xc[q], ax);
-          aw = fma(vc[q], wc[q], aw);
+          const int4 p = pt[32 * k];
+          int h, l;
+          fx_split(vc[32 * k], base, h, l);
+          xx += (long long)h * p.x;
+          xc += (long long)h * p.y;
+          xc += (long long)l * p.x;
+          ww += (long long)h * p.z;
+          wc += (long long)h * p.w;
+          wc += (long long)l * p.z;
         }
-        ax = warp_sum(ax);
-        aw = warp_sum(aw);
-        if (e.lane == 0) {
-          part[c] = ax;
-          part[nd + c] = aw;
+        tx = xx + (xc >> 32);
+        tw = ww + (wc >> 32);
+      };
+      auto put = [&](int c, int isw, long long sum) {
+        const double r = fx_value(sum, fx.ckey[c], isw ? kw : fx.ckey[xout]);
+        part[c == nd ? 2 * nd + isw : isw * nd + c] = r;
+      };
+      if (nd < NW) {               // at most one column per warp
+        if (e.warp <= nd) {
+          long long v[2];
+          dot(e.warp, v[0], v[1]);
+          const long long r = warp_sum_many_s64<2>(v);   // lane l: value l >> 4
+          if ((e.lane & 15) == 0) put(e.warp, e.lane >> 4, r);
         }
-      }
-    } else {                     // all the warp's columns, then one transposed warp sum
-      double v[2 * KMAX];
+      } else {                     // all the warp's columns, then one transposed warp sum
+        long long v[2 * KMAX];
 #pragma unroll
-      for (int kk = 0; kk < KMAX; ++kk) {
-        const int c = e.warp + NW * kk;
-        double ax = 0.0, aw = 0.0;
-        if (c < nd) {
-          const double* vc = Vt + (size_t)c * CL_TP;
-#pragma unroll
-          for (int k = 0; k < CL_TP / 32; ++k) {
-            const int q = e.lane + 32 * k;
-            ax = fma(vc[q], xc[q], ax);
-            aw = fma(vc[q], wc[q], aw);
-          }
+        for (int kk = 0; kk < KMAX; ++kk) {
+          const int c = e.warp + NW * kk;
+          v[2 * kk] = v[2 * kk + 1] = 0;
+          if (c <= nd) dot(c, v[2 * kk], v[2 * kk + 1]);
         }
-        v[2 * kk] = ax;
-        v[2 * kk + 1] = aw;
+        const long long r = warp_sum_many_s64<2 * KMAX>(v);   // lanes 2k, 2k+1: value k
+        const int k = e.lane >> 1, c = e.warp + NW * (k >> 1);
+        if ((e.lane & 1) == 0 && c <= nd) put(c, k & 1, r);
       }
-      const double r = warp_sum_many<2 * KMAX>(v);   // lanes 2k, 2k+1: value k
-      const int k = e.lane >> 1, c = e.warp + NW * (k >> 1);
-      if ((e.lane & 1) == 0 && c < nd) part[(k & 1) ? nd + c : c] = r;
     }
-    if (e.tid < 3) {
+    if (e.tid == 0) {
       double acc = 0.0;
-      for (int i = 0; i < NW; ++i) acc += e.S.bred[i][e.tid];
-      part[2 * nd + e.tid] = acc;
+      for (int i = 0; i < NW; ++i) acc += e.S.bred[i][0];
+      part[stencil ? 2 * nd + 2 : 0] = acc;
     }
     return 2 * nd + 3;
   }
@@ -253,20 +281,21 @@ struct ClusterEngine {
   // holds x_j, the matvec buffers alternate in columns m+1 and m+2.
   __device__ void run_hybrid() {
     const int m = e.P.m, wc = m + 1;
-    if (e.tid == 0) { e.S.a = 1.0; e.S.done = 0; e.S.fallback_pending = 0; e.S.syncs_c = 0; }
+    if (e.tid == 0) { e.S.a = 1.0; e.S.done = 0; e.S.fallback_pending = 0; e.S.syncs_c = 0; fx.wkey = 0; }
+    if (e.tid < MMAX + 2) fx.ckey[e.tid] = 0;
     __syncthreads();
     for (int j = 1; j <= m; ++j) {
       const int ns = pass(j - 1, (j == 1) ? -1 : wc + ((j - 1) & 1), (j == 1) ? 1.0 : (double)e.S.a, j - 1,
-                          wc + (j & 1), SELF_XX | SELF_XW | SELF_WW);
+                          wc + (j & 1));
       reduce(ns, j, [&] { e.hybrid_step(j); });
       if (e.S.done) return;
       if (e.S.fallback_pending) {   // explicit norm of the projected vector (extra reduction)
-        const int nf = pass(j, wc + (j & 1), (double)e.S.a, -1, -1, SELF_XX);
+        const int nf = pass(j, wc + (j & 1), (double)e.S.a, -1, -1);
         reduce(nf, j, [&] { e.hybrid_fallback_finish(j); });
         if (e.S.done) return;
       }
     }
-    const int nl = pass(m, wc + (m & 1), (double)e.S.a, m, -1, SELF_XX);   // v_{m+1} and its norm
+    const int nl = pass(m, wc + (m & 1), (double)e.S.a, m, -1);   // v_{m+1} and its norm
     reduce(nl, 0, [&] { e.hybrid_final_finish(); });
   }
 };
@@ -286,7 +315,8 @@ __global__ void __launch_bounds__(NT, 1) k_arnoldi_cluster(ArnoldiParams P, Smal
   e.gsize = (int)gridDim.x;   // the grid is the cluster
   e.cached = true;            // CTA 0 runs every step: its state stays in shared memory
   ClusterEngine<Op> c(e, reinterpret_cast<double*>(smem_cl + LY::vt_off()),
-                      reinterpret_cast<double*>(smem_cl + LY::part_off(P.m)));
+                      reinterpret_cast<double*>(smem_cl + LY::part_off(P.m)),
+                      *reinterpret_cast<ClusterFix*>(smem_cl + LY::fix_off(P.m)));
   c.run_hybrid();
   __threadfence();   // CTA 0's control block, H and scales, for the exponential
   cl_sync();         // ... and no CTA goes on while another may read its shared memory
