@@ -122,36 +122,33 @@ struct FlatPass {
     }
     const Tc* Vb = reinterpret_cast<const Tc*>(e.P.V);
     int c = ps.c0;
-#pragma unroll 1
-    for (; c + CB <= ps.c1; c += CB) {
-      Tc v[CB][NU][W];
+    // CN columns, their loads before their FMAs (float32: the odd ones of a whole block in the second accumulator)
+    auto block = [&](auto cn) {
+      constexpr int CN = decltype(cn)::value;
+      Tc v[CN][NU][W];
 #pragma unroll
-      for (int k = 0; k < CB; ++k)
+      for (int k = 0; k < CN; ++k)
 #pragma unroll
         for (int u = 0; u < NU; ++u) load<W>(Vb + (long long)(c + k) * N + g[u], v[k][u]);
 #pragma unroll
-      for (int k = 0; k < CB; ++k) {
+      for (int k = 0; k < CN; ++k) {
         const Tc cc = e.S.coefc[c + k];
 #pragma unroll
         for (int u = 0; u < NU; ++u)
 #pragma unroll
           for (int i = 0; i < W; ++i) {
-            if (!F64 && (k & 1)) xb[u][i] = fma(-cc, v[k][u][i], xb[u][i]);
+            if (!F64 && CN == CB && (k & 1)) xb[u][i] = fma(-cc, v[k][u][i], xb[u][i]);
             else x[u][i] = fma(-cc, v[k][u][i], x[u][i]);
           }
       }
-    }
+      c += CN;
+    };
 #pragma unroll 1
-    for (; c < ps.c1; ++c) {
-      const Tc cc = e.S.coefc[c];
-      Tc v[NU][W];
-#pragma unroll
-      for (int u = 0; u < NU; ++u) load<W>(Vb + (long long)c * N + g[u], v[u]);
-#pragma unroll
-      for (int u = 0; u < NU; ++u)
-#pragma unroll
-        for (int i = 0; i < W; ++i) x[u][i] = fma(-cc, v[u][i], x[u][i]);
-    }
+    while (c + CB <= ps.c1) block(std::integral_constant<int, CB>());
+    const int rest = ps.c1 - c;
+    if (rest & 4) block(std::integral_constant<int, 4>());
+    if (rest & 2) block(std::integral_constant<int, 2>());
+    if (rest & 1) block(std::integral_constant<int, 1>());
     unsigned key = 0;
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
