@@ -89,6 +89,7 @@ struct Engine {
   int trow = 0;                      // cached mode: row of T that finish_trow has to form (0: none)
   unsigned bt1 = 0, bt2 = 0;         // arrivals that complete the next waits on the two grid counters
   bool one_level = false;            // batched kernel: order of the float32 form's sums over the CTAs
+  int nrows = 0;                     // rows of partial sums (0: one per CTA)
   int par = 0;                       // buffer of the partial sums (small grids alternate between two)
   Coef<Tc> cf;
   const int tid, lane, warp;
@@ -583,10 +584,12 @@ struct Engine {
 
   __device__ __forceinline__ double* part(int w) const { return small + MMAX * TS + w * 32; }
 
-  // This CTA's row of partial sums.
-  __device__ __forceinline__ double* part_row() const {
-    return (par ? P.gsum : P.partials) + (long long)grank * SLOTS;
+  // A row of partial sums, this CTA's by default.
+  __device__ __forceinline__ double* part_row(int row) const {
+    return (par ? P.gsum : P.partials) + (long long)row * SLOTS;
   }
+  __device__ __forceinline__ double* part_row() const { return part_row(grank); }
+  __device__ __forceinline__ int rows() const { return nrows > 0 ? nrows : gsize; }
 
   // dst[s] = sum of nrows rows of partial sums.  One thread per slot, so the
   // loads of a warp are contiguous; each thread adds its rows in index order,
@@ -690,10 +693,10 @@ struct Engine {
   __device__ bool reduce_all(int nslots, Fn fn) {
     bt1 += (unsigned)gsize;
     if (!arrive_wait(&P.ctl->arrive, bt1, true)) return false;
-    if (gsize <= DIRECT) {
+    if (rows() <= DIRECT) {
       const double* src = par ? P.gsum : P.partials;
-      if constexpr (F64) sum_few(src, gsize, nslots);
-      else sum_few_ordered(src, gsize, nslots);
+      if constexpr (F64) sum_few(src, rows(), nslots);
+      else sum_few_ordered(src, rows(), nslots);
       par ^= 1;
     } else {
       const int nq = (nslots + 3) / 4;
@@ -748,7 +751,7 @@ struct Engine {
   // gsum[s0..s0+3] = the sums of these slots over all rows: thread t takes rows t, t + NT, ...
   __device__ void sum_slots(int s0) {
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int r = tid; r < gsize; r += NT) {
+    for (int r = tid; r < rows(); r += NT) {
       const double2* row = reinterpret_cast<const double2*>(P.partials + (long long)r * SLOTS + s0);
       const double2 a = __ldcg(row), b = __ldcg(row + 1);
       v[0] += a.x; v[1] += a.y; v[2] += b.x; v[3] += b.y;
@@ -779,14 +782,15 @@ struct Engine {
   }
   __device__ double lane_sum(const double* src) const {
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    const int n = rows();
     int c = lane;
-    for (; c + 96 < gsize; c += 128) {
+    for (; c + 96 < n; c += 128) {
       a0 += __ldcg(src + (long long)c * SLOTS);
       a1 += __ldcg(src + (long long)(c + 32) * SLOTS);
       a2 += __ldcg(src + (long long)(c + 64) * SLOTS);
       a3 += __ldcg(src + (long long)(c + 96) * SLOTS);
     }
-    for (; c < gsize; c += 32) a0 += __ldcg(src + (long long)c * SLOTS);
+    for (; c < n; c += 32) a0 += __ldcg(src + (long long)c * SLOTS);
     return warp_sum((a0 + a1) + (a2 + a3));
   }
   __device__ void sum_few_ordered(const double* src, int nrows, int nslots) {
@@ -820,8 +824,8 @@ struct Engine {
       return;
     }
     double* scratch = small + STEP_DOUBLES;
-    const int ngr = (gsize + RG - 1) / RG, s = tid & 3, g = tid >> 2;
-    if (g < ngr) scratch[tid] = run_sum(P.partials + s0 + s, g * RG, min(gsize, (g + 1) * RG));
+    const int ngr = (rows() + RG - 1) / RG, s = tid & 3, g = tid >> 2;
+    if (g < ngr) scratch[tid] = run_sum(P.partials + s0 + s, g * RG, min(rows(), (g + 1) * RG));
     __syncthreads();
     if (tid < 4) {
       double acc = 0.0;
