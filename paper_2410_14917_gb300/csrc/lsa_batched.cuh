@@ -19,6 +19,7 @@
 
 #include "lsa_expm.cuh"
 #include "lsa_flat.cuh"
+#include "lsa_ordered.cuh"
 
 namespace lsa {
 
@@ -99,6 +100,20 @@ __device__ __noinline__ bool batch_arnoldi_flat(const ArnoldiParams& P, int gran
   f.run();
   return batch_results_out(e);
 }
+// (float32: the tile passes' two-phase step with their planes in parallel, single-species operators)
+template <class Op>
+__device__ __noinline__ bool batch_arnoldi_ordered(const ArnoldiParams& P, int grank, int gsize, unsigned char* smem) {
+  using F = OrderedPass<Op>;
+  using E = typename F::E;
+  E e(P, *reinterpret_cast<typename E::Smem*>(smem), reinterpret_cast<double*>(smem + E::small_offset()));
+  e.grank = grank;
+  e.gsize = gsize;
+  e.redundant_steps();
+  e.one_level = true;
+  F f(e, *reinterpret_cast<typename F::Buf*>(smem + F::offset()));
+  f.run();
+  return batch_results_out(e);
+}
 template <class Op, class Tc>
 __device__ __noinline__ bool batch_arnoldi_tiles(const ArnoldiParams& P, int grank, int gsize, unsigned char* smem) {
   using E = Engine<Op, Tc, Tc>;
@@ -163,6 +178,9 @@ __device__ __noinline__ bool batch_instance(const BatchParams& BP, const BatchIn
   bool ok;
   if constexpr (sizeof(Tc) == 8)
     ok = BP.step == 2 && is_hybrid(P.variant) ? batch_arnoldi_flat<Op, Tc>(P, grank, gsize, smem)
+                                              : batch_arnoldi_tiles<Op, Tc>(P, grank, gsize, smem);
+  else if constexpr (Op::NS == 1)
+    ok = BP.step == 1 && is_hybrid(P.variant) ? batch_arnoldi_ordered<Op>(P, grank, gsize, smem)
                                               : batch_arnoldi_tiles<Op, Tc>(P, grank, gsize, smem);
   else
     ok = batch_arnoldi_tiles<Op, Tc>(P, grank, gsize, smem);
@@ -253,7 +271,9 @@ __global__ void __launch_bounds__(NT, 2) k_batched(BatchParams BP) {
 
 template <class Op, class Tc>
 constexpr size_t batched_smem_bytes() {
-  const size_t a = Engine<Op, Tc, Tc>::smem_bytes(), b = sizeof(Tc) == 8 ? FlatPass<Op, Tc>::smem_bytes() : 0;
+  size_t a = Engine<Op, Tc, Tc>::smem_bytes(), b = 0;
+  if constexpr (sizeof(Tc) == 8) b = FlatPass<Op, Tc>::smem_bytes();
+  else if constexpr (Op::NS == 1) b = OrderedPass<Op>::smem_bytes();
   return a > b ? a : b;
 }
 
