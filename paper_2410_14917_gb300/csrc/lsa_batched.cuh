@@ -109,7 +109,6 @@ __device__ __noinline__ bool batch_arnoldi_ordered(const ArnoldiParams& P, int g
   e.grank = grank;
   e.gsize = gsize;
   e.redundant_steps();
-  e.one_level = true;
   F f(e, *reinterpret_cast<typename F::Buf*>(smem + F::offset()));
   f.run();
   return batch_results_out(e);
@@ -121,7 +120,6 @@ __device__ __noinline__ bool batch_arnoldi_tiles(const ArnoldiParams& P, int gra
   e.grank = grank;
   e.gsize = gsize;
   e.redundant_steps();
-  e.one_level = true;
   if (P.variant == LSA_MGS) e.run_mgs(false);
   else if (P.variant == LSA_CGS2) e.run_cgs2(false);
   else if (P.variant == LSA_IOCGS) e.run_iocgs(false);

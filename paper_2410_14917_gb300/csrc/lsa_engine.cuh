@@ -88,7 +88,6 @@ struct Engine {
   bool cached = false, lead = true;
   int trow = 0;                      // cached mode: row of T that finish_trow has to form (0: none)
   unsigned bt1 = 0, bt2 = 0;         // arrivals that complete the next waits on the two grid counters
-  bool one_level = false;            // batched kernel: order of the float32 form's sums over the CTAs
   int nrows = 0;                     // rows of partial sums (0: one per CTA)
   int par = 0;                       // buffer of the partial sums (small grids alternate between two)
   Coef<Tc> cf;
@@ -695,15 +694,11 @@ struct Engine {
     if (!arrive_wait(&P.ctl->arrive, bt1, true)) return false;
     if (rows() <= DIRECT) {
       const double* src = par ? P.gsum : P.partials;
-      if constexpr (F64) sum_few(src, rows(), nslots);
-      else sum_few_ordered(src, rows(), nslots);
+      sum_few(src, rows(), nslots);
       par ^= 1;
     } else {
       const int nq = (nslots + 3) / 4;
-      if (grank < nq) {
-        if constexpr (F64) sum_slots(4 * grank);
-        else sum_slots_ordered(4 * grank);
-      }
+      if (grank < nq) sum_slots(4 * grank);
       bt2 += (unsigned)nq;
       if (!arrive_wait(&P.ctl->release, bt2, grank < nq)) return false;
       for (int s = tid; s < nslots; s += NT) S.red[s] = __ldcg(P.gsum + s);
@@ -762,74 +757,6 @@ struct Engine {
     if (tid < 4) {
       double acc = 0.0;
       for (int i = 0; i < NW; ++i) acc += S.tmp[3][i * 4 + tid];
-      __stcg(P.gsum + s0 + tid, acc);
-    }
-  }
-
-  // The same sums of the float32 form, in one order whatever the reduction's shape (see hybrid_step_ordered):
-  // rows in index order within groups of RG, then the groups; in the batched kernel (one_level) lane by lane.
-  __device__ double run_sum(const double* src, int r0, int r1) const {
-    double acc = 0.0;
-    for (int r = r0; r < r1; r += 16) {
-      double v[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = (r + k < r1) ? __ldcg(src + (long long)(r + k) * SLOTS) : 0.0;
-#pragma unroll
-      for (int k = 0; k < 16; ++k)
-        if (r + k < r1) acc += v[k];
-    }
-    return acc;
-  }
-  __device__ double lane_sum(const double* src) const {
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    const int n = rows();
-    int c = lane;
-    for (; c + 96 < n; c += 128) {
-      a0 += __ldcg(src + (long long)c * SLOTS);
-      a1 += __ldcg(src + (long long)(c + 32) * SLOTS);
-      a2 += __ldcg(src + (long long)(c + 64) * SLOTS);
-      a3 += __ldcg(src + (long long)(c + 96) * SLOTS);
-    }
-    for (; c < n; c += 32) a0 += __ldcg(src + (long long)c * SLOTS);
-    return warp_sum((a0 + a1) + (a2 + a3));
-  }
-  __device__ void sum_few_ordered(const double* src, int nrows, int nslots) {
-    if (one_level) {
-      for (int s = warp; s < nslots; s += NW) {
-        const double v = lane_sum(src + s);
-        if (lane == 0) S.red[s] = v;
-      }
-      return;
-    }
-    static_assert(DIRECT <= 2 * RG, "at most two groups");
-    double* scratch = small + STEP_DOUBLES;
-    const int ngr = (nrows + RG - 1) / RG;
-    for (int i = tid; i < ngr * nslots; i += NT) {
-      const int g = i / nslots, s = i - g * nslots;
-      scratch[g * SLOTS + s] = run_sum(src + s, g * RG, min(nrows, (g + 1) * RG));
-    }
-    __syncthreads();
-    for (int s = tid; s < nslots; s += NT) {
-      double acc = 0.0;
-      for (int g = 0; g < ngr; ++g) acc += scratch[g * SLOTS + s];
-      S.red[s] = acc;
-    }
-  }
-  __device__ void sum_slots_ordered(int s0) {
-    if (one_level) {
-      if (warp < 4) {
-        const double v = lane_sum(P.partials + s0 + warp);
-        if (lane == 0) __stcg(P.gsum + s0 + warp, v);
-      }
-      return;
-    }
-    double* scratch = small + STEP_DOUBLES;
-    const int ngr = (rows() + RG - 1) / RG, s = tid & 3, g = tid >> 2;
-    if (g < ngr) scratch[tid] = run_sum(P.partials + s0 + s, g * RG, min(rows(), (g + 1) * RG));
-    __syncthreads();
-    if (tid < 4) {
-      double acc = 0.0;
-      for (int i = 0; i < ngr; ++i) acc += scratch[4 * i + tid];
       __stcg(P.gsum + s0 + tid, acc);
     }
   }
@@ -906,8 +833,8 @@ struct Engine {
   // waits (finish_trow).  The norm estimate needs t2 only, and one warp forms
   // it beside the others' product with T.
   __device__ void hybrid_step(int j) {
-    if (!F64 || !cached) {
-      hybrid_step_ordered(j);
+    if (!cached) {
+      hybrid_step_last(j);
       return;
     }
     Ctl* ctl = P.ctl;
@@ -1111,10 +1038,8 @@ struct Engine {
     trow = 0;
   }
 
-  // The same step in another order of its sums: the float32 form, and the TMA-staged and streaming kernels
-  // (not cached: run by the CTA that completes the reduction).  A coefficient that rounds the other way to
-  // float32 moves a column by 6e-8, so the float32 form keeps one order of the step's sums.
-  __device__ void hybrid_step_ordered(int j) {
+  // The step of the TMA-staged and streaming kernels (not cached): run by the CTA that completes the reduction.
+  __device__ void hybrid_step_last(int j) {
     Ctl* ctl = P.ctl;
     const int np = j - 1;
     double* temp1 = S.tmp[0];
@@ -1169,7 +1094,7 @@ struct Engine {
     } else {
       // New row of T (Alg. 5: T_{j,1:j-1} = -temp_{1:j-1,1}^T T_{1:j-1,1:j-1};
       // Alg. 6: T_{j,1:j-1} = -temp_{1:j-1,1}^T; for Alg. 7 this is M^{-1}).
-      if (!cached) stage(P.T, np);              // else small already holds rows 0..np-1 of T
+      stage(P.T, np);
       if (P.variant != LSA_HNCWY) {
         // T_{j,k} = -temp1_k - sum_{i>k} temp1_i T_{i,k}: the four lanes
         // 4k..4k+3 (all eight warps) take the terms i = k+1+q, k+5+q, ...
@@ -1184,12 +1109,12 @@ struct Engine {
         if (k < np && q == 0) {
           const double acc = -temp1[k] + a;
           small[np * TS + k] = acc;
-          if (!cached) P.T[np * MMAX + k] = acc;
+          P.T[np * MMAX + k] = acc;
         }
       } else {
         for (int k = tid; k < np; k += NT) {
           small[np * TS + k] = -temp1[k];
-          if (!cached) P.T[np * MMAX + k] = -temp1[k];
+          P.T[np * MMAX + k] = -temp1[k];
         }
       }
       __syncthreads();
@@ -1199,10 +1124,10 @@ struct Engine {
         // Alg. 7: y = M^{-1} temp2; p = (I + N M^{-1}) temp2 = temp2 - L^T y;
         // H_{1:j,j} solves (I + L) x = p.
         apply_unit_lower(temp2, aux, j);                  // aux = y
-        if (!cached) stage(P.L, np);
+        stage(P.L, np);
         for (int k = tid; k < np; k += NT) {
           Lm(np, k) = temp1[k];
-          if (!cached) P.L[np * MMAX + k] = temp1[k];
+          P.L[np * MMAX + k] = temp1[k];
         }
         __syncthreads();
         for (int r = tid; r < j; r += NT) {
@@ -1266,8 +1191,7 @@ struct Engine {
     for (int i = tid; i < j; i += NT) {
       double si = (i == j - 1) ? S.sj : S.sig[i];
       const double c = si * hcol[i] * S.scale;
-      if (cached) S.coefc[i] = (Tc)c;
-      else ctl->coef[i] = c;
+      ctl->coef[i] = c;
     }
   }
 
