@@ -116,7 +116,8 @@ typedef struct {
   float ms_combine;       /* device time of the output combination (phiv only) */
   int launches;           /* kernels this call launched */
   int arnoldi_kernel;     /* Arnoldi kernel that ran: 0 plain loads, 1 TMA-staged tile+halo,
-                             2 streaming (interior-only TMA stages), 3 single thread-block
+                             2 streaming (interior-only TMA stages, or its sums in flat
+                             passes where those are faster), 3 single thread-block
                              cluster, 4 plain loads with the two-phase step, 5 the flat
                              two-phase step (see lsa_tune_step); filled by
                              lsa_arnoldi/lsa_phiv */

@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -27,6 +28,10 @@ cudaError_t launch_arnoldi_flat_grayscott2d_t(const ArnoldiParams&, int, cudaStr
 cudaError_t launch_arnoldi_flat_grayscott2d_frechet(const ArnoldiParams&, int, cudaStream_t);
 cudaError_t launch_arnoldi_ordered_adr3d(const ArnoldiParams&, int, cudaStream_t);
 int ordered_blocks_per_sm_adr3d();
+cudaError_t launch_arnoldi_strip_adr3d(const ArnoldiParams&, int, int, cudaStream_t);
+int strip_blocks_per_sm_adr3d();
+cudaError_t launch_arnoldi_strip_advdiff2d(const ArnoldiParams&, int, int, cudaStream_t);
+int strip_blocks_per_sm_advdiff2d();
 int flat_blocks_per_sm_adr3d(int, int);
 int flat_blocks_per_sm_advdiff2d(int, int);
 int flat_blocks_per_sm_grayscott2d(int, int);
@@ -336,6 +341,25 @@ static int step_form(const ArnoldiParams& P, int precision) {
   return form == 0 ? 0 : 1;
 }
 
+// CTAs of the flat passes with the streaming kernel's sums (lsa_strip.cuh; 0: the streaming kernel itself), among
+// the calls that the streaming kernel takes (LSA_STREAM=1 keeps it for all of them).  Up to 24 columns, or a basis of
+// up to 512 MB, they are faster (ms, streaming kernel and flat passes): 32^3 m = 40 1.21, 0.81; 64^3 m = 40 1.49, 1.03;
+// 128^3 m = 40 5.33, 4.69; 240^3 m = 20 10.5, 8.6; 512^2 1.35, 1.03; 1024^2 2.70, 2.32.  Beyond, the second reading
+// of the basis costs more than the streaming kernel's chain: 192^3 m = 40 13.6, 14.0; 256^3 m = 40 29.9, 31.2; 2048^2
+// m = 40 7.64, 7.96.
+static int strip_grid(const ArnoldiParams& P) {
+  if (P.m > 24 && (size_t)P.op.N * P.m * sizeof(float) > ((size_t)512 << 20)) return 0;
+  const char* env = getenv("LSA_STREAM");
+  if (env && env[0] == '1') return 0;
+  static int cache[2][16];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 16) dev = 0;
+  int& c = cache[P.op.kind == LSA_OP_ADR3D][dev];
+  if (c == 0) c = (P.op.kind == LSA_OP_ADR3D ? strip_blocks_per_sm_adr3d() : strip_blocks_per_sm_advdiff2d()) >= 2 ? 2 : -1;
+  return c < 0 ? 0 : sm_count() * c;
+}
+
 static int arnoldi_kernel_kind(const ArnoldiParams& P, int precision) {
   if (use_cluster(P, precision)) return 3;
   if (use_stream(P, precision)) return 2;
@@ -361,6 +385,11 @@ cudaError_t launch_arnoldi(const ArnoldiParams& P, int precision, int G, cudaStr
 static cudaError_t launch_arnoldi_grid(const ArnoldiParams& P, int precision, int G, cudaStream_t s) {
   if (use_cluster(P, precision)) return launch_arnoldi_cluster_advdiff2d(P, nullptr, nullptr, s);
   if (use_stream(P, precision)) {
+    if (const int F = strip_grid(P)) {
+      const int ranks = std::min(sm_count(), P.tl.ntiles);
+      return P.op.kind == LSA_OP_ADR3D ? launch_arnoldi_strip_adr3d(P, F, ranks, s)
+                                       : launch_arnoldi_strip_advdiff2d(P, F, ranks, s);
+    }
     if (P.op.kind == LSA_OP_ADVDIFF2D) return launch_arnoldi_stream_advdiff2d(P, s);
     return launch_arnoldi_stream_adr3d(P, s);
   }

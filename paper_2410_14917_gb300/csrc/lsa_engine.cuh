@@ -1571,8 +1571,8 @@ __global__ void __launch_bounds__(NT, (sizeof(Tc) == 8) ? LSA_MINB_F64 : LSA_MIN
   else e.run_hybrid();
 }
 
-// y = A x, one thread per grid point (all its species), neighbours through L1; the operator's own arithmetic,
-// so y is bitwise the Arnoldi passes' value.  The float32 form makes its copies of the fields on the fly, so one
+// y = A x, one thread per grid point (all its species), neighbours through L1, with the operator's own
+// arithmetic.  The float32 form makes its copies of the fields on the fly, so one
 // launch does (it was two, the second over persistent CTAs with barriers per tile: 22 us a call on Gray-Scott
 // 512^2, 14.3 us now, launch included).
 template <class Op, class Tc>
