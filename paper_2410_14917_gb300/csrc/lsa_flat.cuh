@@ -123,7 +123,7 @@ struct FlatPass {
     const Tc* Vb = reinterpret_cast<const Tc*>(e.P.V);
     int c = ps.c0;
     // CN columns, their loads before their FMAs (float32: the odd ones of a whole block in the second accumulator)
-    auto block = [&](auto cn) {
+    auto block = [&](auto cn, int c) {
       constexpr int CN = decltype(cn)::value;
       Tc v[CN][NU][W];
 #pragma unroll
@@ -141,14 +141,20 @@ struct FlatPass {
             else x[u][i] = fma(-cc, v[k][u][i], x[u][i]);
           }
       }
-      c += CN;
     };
 #pragma unroll 1
-    while (c + CB <= ps.c1) block(std::integral_constant<int, CB>());
-    const int rest = ps.c1 - c;
-    if (rest & 4) block(std::integral_constant<int, 4>());
-    if (rest & 2) block(std::integral_constant<int, 2>());
-    if (rest & 1) block(std::integral_constant<int, 1>());
+    for (; c + CB <= ps.c1; c += CB) block(std::integral_constant<int, CB>(), c);
+    // the last columns: blocks of four, two and one (Gray-Scott 512^2 5.66 to 5.62 ms, ADR 256^3 54.97 to 53.82); the
+    // augmented kernel, with less registers to spare, takes them one by one (6.84 ms in blocks, 6.64 so)
+    if constexpr (AUG) {
+#pragma unroll 1
+      for (; c < ps.c1; ++c) block(std::integral_constant<int, 1>(), c);
+    } else {
+      const int rest = ps.c1 - c;
+      if (rest & 4) block(std::integral_constant<int, 4>(), c);
+      if (rest & 2) block(std::integral_constant<int, 2>(), c + (rest & 4));
+      if (rest & 1) block(std::integral_constant<int, 1>(), c + (rest & 6));
+    }
     unsigned key = 0;
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
