@@ -47,11 +47,13 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # Arnoldi kernel kind (0 one-pass, 4 two-phase grid kernel, 5 flat two-phase
 # kernel, 2 streaming);
 # a workload without an up-to-date capture reports null.  Gray-Scott 512^2:
-# profiles/k_arnoldi_grayscott2d_512_fp64.md (both step forms); the 3D line's
+# profiles/k_arnoldi_grayscott2d_512_fp64.md (both tile step forms) and
+# profiles/k_arnoldi_flat_grayscott2d_512_fp64.md (flat); the 3D line's
 # capture is of the 192^3 case (same tiling), scaled by the unknowns
 # ((256/192)^3) (profiles/k_arnoldi_stream_adr3d_192_fp32.md).
 PROFILED_TRAFFIC = {("grayscott2d_512", "fp64", "hcwy", 0): 9.118409e9 + 0.744297e9,
                     ("grayscott2d_512", "fp64", "hcwy", 4): 13.717263e9 + 0.777655e9,
+                    ("grayscott2d_512", "fp64", "hcwy", 5): 17.076877e9 + 0.787758e9,
                     ("adr3d_256", "fp32", "hcwy", 2): (28.712327e9 + 2.551436e9) * (256 / 192) ** 3}
 
 

@@ -20,8 +20,8 @@
 // which a warp keeps 6 KB in flight (in registers, 2 to 4 KB: ADR 256^3 70 against
 // 73 ms a phi product; with the limbs kept instead of converted 56 ms; the float64
 // products it replaces took 94).  It walks its share backwards, so that it
-// starts on the columns' values that pass A left in L2, and the next pass A on
-// those that pass B left.
+// starts on the x that pass A left in L2 (and, where the columns are converted in
+// place, on theirs).
 #pragma once
 
 #include <type_traits>
