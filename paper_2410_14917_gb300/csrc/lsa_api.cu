@@ -191,8 +191,9 @@ static bool use_tma(const ArnoldiParams& P, int precision) {
 
 // The streaming kernel (interior-only TMA stages, halo by plain loads) runs
 // the hybrid variants of the float32-basis form for the single-species
-// operators whenever its stages fit (LSA_STREAM=0 in the environment disables
-// it; the other kernels then run).
+// operators whenever its stages fit, itself or by flat passes with its sums
+// (strip_grid) (LSA_STREAM=0 in the environment disables both; the other
+// kernels then run).
 static bool use_stream(const ArnoldiParams& P, int precision) {
   if (!is_hybrid(P.variant) || precision != LSA_FP32_BASIS || !P.E || P.naug > 0) return false;
   const char* env = getenv("LSA_STREAM");
@@ -299,10 +300,10 @@ static int flat_ctas_per_sm(const ArnoldiParams& P, int precision) {
 
 // Where nothing is recorded or forced, the flat kernel runs
 //  * in float64 at every size (a phi product on GB300, flat against one-pass:
-//    Gray-Scott 48^2 0.61 and 0.80 ms, 256^2 1.7 and 2.1, 512^2 5.7 and 9.6;
+//    Gray-Scott 48^2 0.61 and 0.80 ms, 256^2 1.7 and 2.1, 512^2 5.6 and 9.6;
 //    advection-diffusion 97 x 61 0.41 and 0.46; ADR 16^3 0.36 and 0.82);
 //  * with the float32 basis on 2D grids of at least six 16 x 16 tiles per SM
-//    (Gray-Scott 512^2 2.6 against 4.4 ms; below that, and on 3D grids that the
+//    (Gray-Scott 512^2 2.1 against 4.4 ms; below that, and on 3D grids that the
 //    streaming and TMA-staged kernels do not take, the tile forms).
 static bool flat_default(const ArnoldiParams& P, int precision) {
   if (!is_hybrid(P.variant) || flat_ctas_per_sm(P, precision) == 0) return false;
@@ -318,7 +319,7 @@ static int flat_grid(const ArnoldiParams& P, int precision) {
 
 // CTAs of the float32 3D two-phase kernel with the tile passes' sums (lsa_ordered.cuh; 0: another operator, form
 // or precision).  It repeats the tile passes' results to the last bit and is faster at every size tried: 75 x 50 x 41
-// 3.20 to 0.60 ms, 30 x 20 x 90 1.20 to 0.73, 150 x 100 x 70 5.40 to 2.39, 210 x 200 x 190 20.5 to 13.2, 64^3 2.17
+// 3.20 to 0.55 ms, 30 x 20 x 90 1.20 to 0.73, 150 x 100 x 70 5.40 to 2.39, 210 x 200 x 190 20.5 to 13.2, 64^3 2.17
 // to 1.29.  (In 2D a tile is one plane and the tile passes use the whole GPU: 1.19 ms at 256^2 against 1.29.)
 static int ordered_grid(const ArnoldiParams& P, int precision) {
   if (P.two_phase != 1 || precision != LSA_FP32_BASIS || P.op.kind != LSA_OP_ADR3D || !is_hybrid(P.variant)) return 0;

@@ -19,7 +19,7 @@
 // before their FMAs (with one point a thread and the last columns one by one it
 // took 1.25 times as long), pass B2 four columns of a plane.  Sixteen columns a
 // unit, so that x and w are read again once every sixteen columns.  A step of
-// 75 x 50 x 41 (m = 20) takes 24 us, of which the passes are 8, the barriers 8
+// 75 x 50 x 41 (m = 20) takes 22 us, of which the passes are 8, the barriers 8
 // and the reduction and step function the rest.
 #pragma once
 
