@@ -48,12 +48,18 @@ __device__ __forceinline__ void fx_split0(double v, unsigned base, int& h, int& 
   if (fx_key(v) < 0x100000u) h = l = 0;
 }
 
+// 2^(E - 26) for a block of largest key k: half the scale of a product's sum, so that neither half leaves the range
+// of float64 before the product does.  0 for a block of zeros and subnormal values.
+__device__ __forceinline__ double fx_scale(unsigned k) {
+  const int e = (int)(k >> 20) - 26;                                  // biased exponent
+  if (k < 0x100000u) return 0.0;
+  return e > 0 ? __hiloint2double(e << 20, 0) : __longlong_as_double(1LL << (51 + e));
+}
+
 // sum 2^(Ev + Ex - 52): a sum of products (in units of 2^64 limb units) of blocks with the largest keys kv and
-// kx.  Below 2^-960 it is flushed to zero.
+// kx.  It underflows where the float64 products would: the squares of a start vector of 1e-150 count.
 __device__ __forceinline__ double fx_value(long long sum, unsigned kv, unsigned kx) {
-  const int w = (int)(kv >> 20) + (int)(kx >> 20) - (1023 + 52);      // biased exponent of the unit
-  const double unit = w <= 0 ? 0.0 : __hiloint2double((w < 2046 ? w : 2046) << 20, 0);
-  return (double)sum * unit;
+  return (double)sum * fx_scale(min(kv, kx)) * fx_scale(max(kv, kx));
 }
 
 // Warp sums of NV 64-bit integers at once (warp_sum_many's scheme): lane l gets the sum of value

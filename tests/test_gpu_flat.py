@@ -123,3 +123,41 @@ def test_flat_without_room_for_the_limbs(nx, ny, m):
     y, st = _forced(2, lambda: lsa.phiv_noalloc(op, v, 1e-2, 1, m))
     assert st["m_eff"] == m
     assert float((y - ref).norm()) <= 1e-12 * float(ref.norm())
+
+
+@pytest.mark.parametrize("path", ["flat", "flat_in_place", "cluster", "batch"])
+@pytest.mark.parametrize("bits", [-500, -505, 490])
+def test_start_vectors_near_the_ends_of_the_range(path, bits):
+    """v scaled by a power of two whose square is still a float64 gives the
+    same products scaled: rounding is the same, and what underflows in the
+    sums is 2^-1074 a value against squares above 2^-1010, so the two agree
+    far below 1e-14."""
+    import paper_2410_14917_gb300 as lsa
+
+    n = 64 if path == "cluster" else 201
+    cfg = W.advdiff2d(n, ny=n, m=20, p=1)
+    op, v = _op(cfg)
+
+    def call(x):
+        if path == "batch":
+            b = lsa.Batch([op], [20], 1e-2, 1)
+            y = b.run(x).clone().view(2, -1)
+            st, fin, _ = b.stats()
+            assert st >= 0 and fin == 1
+            b.close()
+            return y
+        if path == "cluster":
+            y, st = lsa.phiv(op, x, 1e-2, 1, 20)
+            assert st["arnoldi_kernel"] == 3
+        elif path == "flat":
+            y, st = _forced(2, lambda: lsa.phiv(op, x, 1e-2, 1, 20))
+            assert st["arnoldi_kernel"] == 5
+        else:
+            w = lsa.Workspace.for_call(op, 20, 1)
+            w.nbytes -= 256                  # ends inside the fixed-point basis
+            y, st = _forced(2, lambda: lsa.phiv(op, x, 1e-2, 1, 20, work=w))
+        assert st["m_eff"] == 20
+        return y
+
+    ref, y = call(v), call(v * 2.0**bits)
+    assert float((y * 2.0**-bits - ref).norm()) <= 1e-14 * float(ref.norm())
