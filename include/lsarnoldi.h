@@ -138,7 +138,7 @@ long long lsa_op_dof(const lsa_op* op);
 /* Bytes of device workspace needed by lsa_phiv / lsa_arnoldi for (op, m, p,
  * precision) on the current device; 0 if the arguments are invalid.  The
  * workspace must be 256-byte aligned.  Its contents need not be initialised.
- * In float64 it ends with a second, fixed-point copy of the basis (8 N m bytes,
+ * In float64 it ends with a second, fixed-point copy of the basis (8 N m bytes and a 64th,
  * up to 64 GiB), which the flat kernel's inner products read; the calls also
  * take a workspace without that part and then convert the columns at each use. */
 size_t lsa_workspace_bytes(const lsa_op* op, int m, int p, int precision);

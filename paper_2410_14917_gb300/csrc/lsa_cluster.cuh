@@ -23,7 +23,7 @@
 //
 //  * the pass's inner products, two FMAs per column value and bound by the
 //    float64 unit of its 16 SMs, are exact integer sums instead (lsa_fix.cuh):
-//    64 x 64 with m = 30 takes 344 us a phi product, 405 with float64 products.
+//    64 x 64 with m = 30 takes 358 us a phi product, 405 with float64 products.
 //
 // Per Alg. 4 step: three cluster barriers (halo ready, partials ready, step
 // published) and no global-memory barrier.  The hardware cluster barrier has
@@ -72,12 +72,12 @@ __device__ __forceinline__ void cl_st(int* local, unsigned rank, int v) {
 // of the O(j^2) step, which holds T, and GSMGS's L, between steps in CTA 0):
 // the tile's basis [m+3][CL_TP] (columns 0..m, then the two
 // matvec buffers m+1, m+2) and the CTA's partial sums [SLOTS].
-// The tile's x and w as limbs (xh, xl, wh, wl), and the largest keys of its slice of every column and of w
-// (lsa_fix.cuh).
+// The tile's x and w as limbs (xh, xl, wh, wl), the shift bases of its slice of every column, and the warps' largest
+// keys and sums of squares of x and w (lsa_fix.cuh).
 struct ClusterFix {
   int4 xw[CL_TP];
   unsigned ckey[MMAX + 2];
-  unsigned wkey;
+  uint2 blk[2 * NW];
 };
 
 template <class Op>
@@ -127,6 +127,21 @@ struct ClusterEngine {
     return r == e.grank ? *p : cl_ld(p, (unsigned)r);
   }
 
+  // The warp's share of a block's scale, and the scales of the tile's x and w from its warps' shares.
+  __device__ __forceinline__ void warp_block(double v, uint2& out) const {
+    const unsigned k = __reduce_max_sync(0xffffffffu, fx_key(v));
+    const unsigned q = __reduce_add_sync(0xffffffffu, fx_square(v, k));
+    if (e.lane == 0) out = make_uint2(k, q);
+  }
+  __device__ __forceinline__ void tile_bases(unsigned& bx, unsigned& bw) const {
+    const uint2 x = fx.blk[e.lane & (NW - 1)], w = fx.blk[NW + (e.lane & (NW - 1))];
+    const unsigned kx = __reduce_max_sync(0xffffffffu, x.x), kw = __reduce_max_sync(0xffffffffu, w.x);
+    const unsigned qx = e.lane < NW ? x.y >> min(2u * (((kx | 0xfffffu) - x.x) >> 20), 31u) : 0u;
+    const unsigned qw = e.lane < NW ? w.y >> min(2u * (((kw | 0xfffffu) - w.x) >> 20), 31u) : 0u;
+    bx = fx_base(kx, __reduce_add_sync(0xffffffffu, qx));
+    bw = fx_base(kw, __reduce_add_sync(0xffffffffu, qw));
+  }
+
   // One pass of the hybrid process over this tile: x = a*src - sum_{c < ncp}
   // coef_c V_c (src < 0: the start vector), stored in column xout (>= 0); with
   // wout >= 0 the stencil w = A x into column wout and the inner products of
@@ -151,8 +166,7 @@ struct ClusterEngine {
     }
     double w = 0.0;
     if (stencil) {
-      const unsigned kx = __reduce_max_sync(0xffffffffu, fx_key(x));
-      if (e.lane == 0) atomicMax(&fx.ckey[xout], kx);     // (zeroed by run_hybrid)
+      warp_block(x, fx.blk[e.warp]);
       cl_sync();   // every tile's x is in its CTA's shared memory
       const Coef<double>& cf = e.cf;
       double r = cf.cC * x;
@@ -162,8 +176,7 @@ struct ClusterEngine {
       r = fma(cf.cN, (ly < TY - 1) ? Vt[(size_t)xout * CL_TP + t + TX] : xat(xout, gx, gy + 1), r);
       w = r;
       Vt[(size_t)wout * CL_TP + t] = w;
-      const unsigned kw = __reduce_max_sync(0xffffffffu, fx_key(w));
-      if (e.lane == 0) atomicMax(&fx.wkey, kw);
+      warp_block(w, fx.blk[NW + e.warp]);
     }
     // self term in float64 (the others are inner products with column xout): warp sums
     {
@@ -173,37 +186,33 @@ struct ClusterEngine {
     __syncthreads();   // x, w, their keys and the warp sums are in shared memory
     const int nd = stencil ? ncp : 0;
     if (stencil) {
-      const unsigned kw = fx.wkey;
+      unsigned kx, kw;
+      tile_bases(kx, kw);
       int4 q;
-      fx_split0(x, fx_base(fx.ckey[xout]), q.x, q.y);
-      fx_split0(w, fx_base(kw), q.z, q.w);
+      fx_split(x, kx, q.x, q.y);
+      fx_split(w, kw, q.z, q.w);
       fx.xw[t] = q;
+      if (t == 0) fx.ckey[xout] = kx;
       __syncthreads();
-      if (t == 0) fx.wkey = 0;
       // inner products on the integer unit (lsa_fix.cuh): warp <-> columns c = warp, warp + NW, ... <= nd (the
       // last one is x), lane <-> points
       auto dot = [&](int c, long long& tx, long long& tw) {
+        constexpr int VL = CL_TP / 32;
         const double* vc = Vt + (size_t)c * CL_TP + e.lane;
         const int4* pt = fx.xw + e.lane;
-        const unsigned base = fx_base(fx.ckey[c]);
-        long long xx = 0, xc = 1LL << 31, ww = 0, wc = 1LL << 31;
+        int h[VL], l[VL], xh[VL], xl[VL], wh[VL], wl[VL];
 #pragma unroll
-        for (int k = 0; k < CL_TP / 32; ++k) {
+        for (int k = 0; k < VL; ++k) {
           const int4 p = pt[32 * k];
-          int h, l;
-          fx_split(vc[32 * k], base, h, l);
-          xx += (long long)h * p.x;
-          xc += (long long)h * p.y;
-          xc += (long long)l * p.x;
-          ww += (long long)h * p.z;
-          wc += (long long)h * p.w;
-          wc += (long long)l * p.z;
+          xh[k] = p.x; xl[k] = p.y; wh[k] = p.z; wl[k] = p.w;
         }
-        tx = xx + (xc >> 32);
-        tw = ww + (wc >> 32);
+        const unsigned base = fx.ckey[c];
+#pragma unroll
+        for (int k = 0; k < VL; ++k) fx_split(vc[32 * k], base, h[k], l[k]);
+        fx_dot(h, l, xh, xl, wh, wl, c == nd, tx, tw);
       };
       auto put = [&](int c, int isw, long long sum) {
-        const double r = fx_value(sum, fx.ckey[c], isw ? kw : fx.ckey[xout]);
+        const double r = fx_value(sum, fx.ckey[c], isw ? kw : kx);
         part[c == nd ? 2 * nd + isw : isw * nd + c] = r;
       };
       if (nd < NW) {               // at most one column per warp
@@ -281,8 +290,7 @@ struct ClusterEngine {
   // holds x_j, the matvec buffers alternate in columns m+1 and m+2.
   __device__ void run_hybrid() {
     const int m = e.P.m, wc = m + 1;
-    if (e.tid == 0) { e.S.a = 1.0; e.S.done = 0; e.S.fallback_pending = 0; e.S.syncs_c = 0; fx.wkey = 0; }
-    if (e.tid < MMAX + 2) fx.ckey[e.tid] = 0;
+    if (e.tid == 0) { e.S.a = 1.0; e.S.done = 0; e.S.fallback_pending = 0; e.S.syncs_c = 0; }
     __syncthreads();
     for (int j = 1; j <= m; ++j) {
       const int ns = pass(j - 1, (j == 1) ? -1 : wc + ((j - 1) & 1), (j == 1) ? 1.0 : (double)e.S.a, j - 1,

@@ -55,15 +55,13 @@ struct FlatPass {
   static constexpr int NGRP = MMAX / FLAT_CG;
   static_assert(FLAT_CG == 8, "the transposed warp sums below take 16 values");
 
-  // Shared memory after the engine's.  float64: the warps' inner products, the
-  // largest keys of this share of the columns (lsa_fix.cuh) and the rings of
-  // columns in flight; float32: every lane's Kahan pairs and the chunk's x and
+  // Shared memory after the engine's.  float64: the warps' inner products and the
+  // rings of columns in flight; float32: every lane's Kahan pairs and the chunk's x and
   // w.  And the stencil's coefficients, converted once: in registers the
   // compiler converts them again at every use, on the float64 pipe.
   struct Buf64 {
     alignas(16) unsigned char ring[NW][FLAT_RING];
     double sum[NW][NGRP * 16];
-    unsigned ckey[MMAX + 2];
     Coef<double> cf;
   };
   struct Buf32 {
@@ -88,9 +86,6 @@ struct FlatPass {
     e1 = min(np, e0 + per);
     vec = np % VW == 0 && ((size_t)e.P.V & 15) == 0;
     if (e.tid == 0) b.cf = e.cf;
-    if constexpr (F64) {
-      if (e.tid < MMAX + 2) b.ckey[e.tid] = 0;
-    }
     __syncthreads();
   }
 
@@ -98,9 +93,9 @@ struct FlatPass {
   // Pass A on `NU` units of one thread: unit u is VW consecutive values at
   // g[u] (32 lanes: 32 VW values).  Columns in ascending order with one
   // accumulator per value (float32: two, alternating), CB columns' loads in
-  // flight before their FMAs.  Returns the largest key of the values.
+  // flight before their FMAs.
   template <int W, int NU>
-  __device__ __forceinline__ unsigned project_units(const PassT<Tc>& ps, const long long (&g)[NU], const bool (&on)[NU]) {
+  __device__ __forceinline__ void project_units(const PassT<Tc>& ps, const long long (&g)[NU], const bool (&on)[NU]) {
     constexpr int CB = 8;
     const long long N = e.P.op.N;
     const Tc a = (Tc)ps.a;
@@ -155,19 +150,16 @@ struct FlatPass {
       if (rest & 2) block(std::integral_constant<int, 2>(), c + (rest & 4));
       if (rest & 1) block(std::integral_constant<int, 1>(), c + (rest & 6));
     }
-    unsigned key = 0;
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
       if (!on[u]) continue;
 #pragma unroll
       for (int i = 0; i < W; ++i) {
         if (!F64) x[u][i] += xb[u][i];
-        else key = max(key, fx_key(x[u][i]));
         if (ps.self & SELF_XX) e.self_add(0, x[u][i], x[u][i]);
       }
       if (ps.xout) store<W>(ps.xout + g[u], x[u]);
     }
-    return key;
   }
 
   template <int W>
@@ -192,7 +184,7 @@ struct FlatPass {
   // turn, two at a time, so that the tail of a short share leaves whole warps
   // without work instead of lanes.
   template <int W>
-  __device__ __forceinline__ unsigned project_w(const PassT<Tc>& ps) {
+  __device__ __forceinline__ void project_w(const PassT<Tc>& ps) {
     constexpr int UW = 32 * W;
     const int cnt = (int)(e1 - e0);
     const int per = (cnt + UW - 1) / UW, units = NS * per;
@@ -204,27 +196,21 @@ struct FlatPass {
       return sp * np + e0 + (on ? q : 0);
     };
     int u = e.warp;
-    unsigned key = 0;
 #pragma unroll 1
     for (; u + NW < units; u += 2 * NW) {
       bool on[2];
       const long long g[2] = {at(u, on[0]), at(u + NW, on[1])};
-      key = max(key, project_units<W, 2>(ps, g, on));
+      project_units<W, 2>(ps, g, on);
     }
     if (u < units) {
       bool on[1];
       const long long g[1] = {at(u, on[0])};
-      key = max(key, project_units<W, 1>(ps, g, on));
+      project_units<W, 1>(ps, g, on);
     }
-    return key;
   }
-  // (col: the column that x becomes, for the key of this share of it, or -1)
-  __device__ void project(const PassT<Tc>& ps, int col) {
-    unsigned key = vec ? project_w<VW>(ps) : project_w<1>(ps);
-    if constexpr (F64) {
-      key = __reduce_max_sync(0xffffffffu, key);
-      if (col >= 0 && e.lane == 0) atomicMax(&b.ckey[col], key);
-    }
+  __device__ void project(const PassT<Tc>& ps) {
+    if (vec) project_w<VW>(ps);
+    else project_w<1>(ps);
   }
 
   // -------------------------------------------------------------------------
@@ -284,29 +270,19 @@ struct FlatPass {
     }
   }
 
-  // Sums of the products of the limbs (h, l) of a column with those of x and w, in units of 2^64 limb units.
+  // x . x and x . w of a piece, as the inner products of column nv (x itself).
   template <int VL>
-  __device__ __forceinline__ static void fx_dot(const int (&h)[VL], const int (&l)[VL], const int (&xh)[VL],
-                                                const int (&xl)[VL], const int (&wh)[VL], const int (&wl)[VL],
-                                                long long& tx, long long& tw) {
-    static_assert(VL <= 8, "a warp's sums stay below 2^62");
-    long long xx = 0, xc = 1LL << 31, ww = 0, wc = 1LL << 31;
-#pragma unroll
-    for (int k = 0; k < VL; ++k) {
-      xx += (long long)h[k] * xh[k];
-      xc += (long long)h[k] * xl[k];
-      xc += (long long)l[k] * xh[k];
-      ww += (long long)h[k] * wh[k];
-      wc += (long long)h[k] * wl[k];
-      wc += (long long)l[k] * wh[k];
-    }
-    tx = xx + (xc >> 32);
-    tw = ww + (wc >> 32);
+  __device__ __forceinline__ void self_products(const int (&xh)[VL], const int (&xl)[VL], const int (&wh)[VL],
+                                                const int (&wl)[VL], unsigned kx, unsigned kw, int nv) {
+    long long t[2];
+    fx_dot(xh, xl, xh, xl, wh, wl, true, t[0], t[1]);
+    const long long s = warp_sum_many_s64<2>(t);         // lane l: value l >> 4
+    if ((e.lane & 15) == 0) b.sum[e.warp][2 * nv + (e.lane >> 4)] += fx_value(s, kx, e.lane ? kw : kx);
   }
 
   // One piece of pass B with the limbs of the basis kept in P.F: lane l takes the VP points
-  // p0 + 2 l + 64 k + {0, 1} of the share.  Pass B of step j writes the limbs of x_j, in blocks of the CTA's
-  // share, and every later step reads them: eight bytes a value like the float64 column, 16-byte copies at any
+  // p0 + 2 l + 64 k + {0, 1} of the share.  Pass B of step j writes the limbs of x_j and the shift base of each of
+  // its pieces, and every later step reads them: eight bytes a value like the float64 column, 16-byte copies at any
   // N (the columns of F are padded), and no conversion, which takes three times the multiply-adds' time.
   template <int VP>
   __device__ __forceinline__ void piece_fixed(const PassT<Tc>& ps, int p0, int nc, int cs, int CS) {
@@ -339,10 +315,10 @@ struct FlatPass {
 #pragma unroll
     for (int i = 0; i < D; ++i) issue();
     int xh[VL], xl[VL], wh[VL], wl[VL];
-    const unsigned kx = b.ckey[nv];
-    unsigned kw = 0;
+    unsigned* const keys = limb_keys(e.P.F, e.P.op, e.P.m) + (e0 + p0) / 32 * limb_key_stride(e.P.m);
+    unsigned kx, kw;
     {
-      double w[VL];
+      double x[VL], w[VL];
       constexpr int GB = VP < 4 ? VP : 4;            // points whose loads are in flight together
 #pragma unroll
       for (int k0 = 0; k0 < VP; k0 += GB) {
@@ -366,21 +342,34 @@ struct FlatPass {
           for (int sp = 0; sp < NS; ++sp) {
             const int v = sp * VP + k0 + i;
             w[v] = wv[sp];
-            fx_split0(in[i] ? n[i].c5[5 * sp + 2] : 0.0, fx_base(kx), xh[v], xl[v]);
-            if (in[i] && cs == 0)
-              mine[nv * NF + sp * npf + 64 * ((k0 + i) / 2) + (i & 1)] = make_int2(xl[v], xh[v]);
+            x[v] = in[i] ? n[i].c5[5 * sp + 2] : 0.0;
           }
         }
       }
+      fx_blocks(x, w, kx, kw);
 #pragma unroll
-      for (int v = 0; v < VL; ++v) kw = max(kw, fx_key(w[v]));
-      kw = __reduce_max_sync(0xffffffffu, kw);
+      for (int v = 0; v < VL; ++v) {
+        fx_split(x[v], kx, xh[v], xl[v]);
+        fx_split(w[v], kw, wh[v], wl[v]);
+      }
+      if (cs == 0) {
+        // (two points a store: a share ends at an even point, or at the last one and its padding)
+        if (e.lane == 0) keys[nv] = kx;
 #pragma unroll
-      for (int v = 0; v < VL; ++v) fx_split0(w[v], fx_base(kw), wh[v], wl[v]);
+        for (int k = 0; k < VP; k += 2)
+          if (p0 + 2 * e.lane + 32 * k < cnt)
+#pragma unroll
+            for (int sp = 0; sp < NS; ++sp) {
+              const int v = sp * VP + k;
+              *reinterpret_cast<int4*>(mine + nv * NF + sp * npf + 32 * k) = make_int4(xl[v], xh[v], xl[v + 1], xh[v + 1]);
+            }
+      }
     }
+    if (cs == 0) self_products<VL>(xh, xl, wh, wl, kx, kw, nv);
 #pragma unroll 1
-    for (int g = cs; g * FLAT_CG < nc; g += CS) {
-      const int c0 = g * FLAT_CG;
+    for (int g = cs; g * FLAT_CG < nv; g += CS) {
+      const int c0 = g * FLAT_CG, kc = c0 + (e.lane >> 2);
+      const unsigned kv = kc < nv ? __ldcg(keys + kc) : kx;    // of the column whose sum this lane gets
       long long t[16];
 #pragma unroll
       for (int i = 0; i < FLAT_CG; ++i) {
@@ -399,17 +388,14 @@ struct FlatPass {
                            : "r"(rd + (sp * (VP / 2) + k) * 512)
                            : "memory");
             }
-          fx_dot<VL>(h, l, xh, xl, wh, wl, t[2 * i], t[2 * i + 1]);
-        } else if (c == nv) {
-          fx_dot<VL>(xh, xl, xh, xl, wh, wl, t[2 * i], t[2 * i + 1]);
+          fx_dot(h, l, xh, xl, wh, wl, false, t[2 * i], t[2 * i + 1]);
         }
         rd = rd == ring + (D - 1) * CB ? ring : rd + CB;
         issue();
       }
       const long long s = warp_sum_many_s64<16>(t);      // lanes 2k, 2k + 1: value k
-      const int c = min(c0 + (e.lane >> 2), nv);
       if ((e.lane & 1) == 0)
-        b.sum[e.warp][g * 16 + (e.lane >> 1)] += fx_value(s, b.ckey[c], (e.lane & 2) ? kw : kx);
+        b.sum[e.warp][g * 16 + (e.lane >> 1)] += fx_value(s, kv, (e.lane & 2) ? kw : kx);
     }
     flat_wait<0>();        // (columns beyond the last group: nothing in flight into the next piece's slots)
   }
@@ -456,11 +442,10 @@ struct FlatPass {
 #pragma unroll
     for (int i = 0; i < D; ++i) issue();
     int xh[VL], xl[VL], wh[VL], wl[VL];
-    const unsigned kx = b.ckey[nv];
-    unsigned kw = 0;
+    unsigned kx, kw;
     {
       Nbr n[VP];
-      double w[VL];
+      double x[VL], w[VL];
 #pragma unroll
       for (int k = 0; k < VP; ++k) gather(ps.srcB, q[k], n[k]);
 #pragma unroll
@@ -473,44 +458,49 @@ struct FlatPass {
         for (int sp = 0; sp < NS; ++sp) {
           const int v = sp * VP + k;
           w[v] = wv[sp];
-          fx_split0(in[k] ? n[k].c5[5 * sp + 2] : 0.0, fx_base(kx), xh[v], xl[v]);
+          x[v] = in[k] ? n[k].c5[5 * sp + 2] : 0.0;
         }
       }
+      fx_blocks(x, w, kx, kw);
 #pragma unroll
-      for (int v = 0; v < VL; ++v) kw = max(kw, fx_key(w[v]));
-      kw = __reduce_max_sync(0xffffffffu, kw);
-#pragma unroll
-      for (int v = 0; v < VL; ++v) fx_split0(w[v], fx_base(kw), wh[v], wl[v]);
+      for (int v = 0; v < VL; ++v) {
+        fx_split(x[v], kx, xh[v], xl[v]);
+        fx_split(w[v], kw, wh[v], wl[v]);
+      }
     }
+    if (cs == 0) self_products<VL>(xh, xl, wh, wl, kx, kw, nv);
 #pragma unroll 1
-    for (int g = cs; g * FLAT_CG < nc; g += CS) {
+    for (int g = cs; g * FLAT_CG < nv; g += CS) {
       const int c0 = g * FLAT_CG;
       long long t[16];
+      unsigned kv = kx;                                  // of the column whose sum this lane gets
 #pragma unroll
       for (int i = 0; i < FLAT_CG; ++i) {
         const int c = c0 + i;
         t[2 * i] = t[2 * i + 1] = 0;
         if (c < nv) {
-          const unsigned base = fx_base(b.ckey[c]);
+          double v[VL];
           int h[VL], l[VL];
           flat_wait<D - 1>();
 #pragma unroll
-          for (int k = 0; k < VL; ++k) {
-            double v;
-            asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(rd + k * 256) : "memory");
-            fx_split(v, base, h[k], l[k]);
-          }
-          fx_dot<VL>(h, l, xh, xl, wh, wl, t[2 * i], t[2 * i + 1]);
-        } else if (c == nv) {
-          fx_dot<VL>(xh, xl, xh, xl, wh, wl, t[2 * i], t[2 * i + 1]);
+          for (int k = 0; k < VL; ++k) asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v[k]) : "r"(rd + k * 256) : "memory");
+#pragma unroll
+          for (int k = 0; k < VP; ++k)
+            if (!in[k])                                  // (a copy of another point: not in the block)
+#pragma unroll
+              for (int sp = 0; sp < NS; ++sp) v[sp * VP + k] = 0.0;
+          const unsigned kc = fx_block(v);
+          if (e.lane >> 2 == i) kv = kc;
+#pragma unroll
+          for (int k = 0; k < VL; ++k) fx_split(v[k], kc, h[k], l[k]);
+          fx_dot(h, l, xh, xl, wh, wl, false, t[2 * i], t[2 * i + 1]);
         }
         rd = rd == ring + (D - 1) * CB ? ring : rd + CB;
         issue();
       }
       const long long s = warp_sum_many_s64<16>(t);
-      const int c = min(c0 + (e.lane >> 2), nv);
       if ((e.lane & 1) == 0)
-        b.sum[e.warp][g * 16 + (e.lane >> 1)] += fx_value(s, b.ckey[c], (e.lane & 2) ? kw : kx);
+        b.sum[e.warp][g * 16 + (e.lane >> 1)] += fx_value(s, kv, (e.lane & 2) ? kw : kx);
     }
     flat_wait<0>();
   }
@@ -684,7 +674,7 @@ struct FlatPass {
       ps.d0 = ps.d1 = 0;
       ps.self = 0;
       if constexpr (AUG) e.aug_begin(ps);
-      project(ps, j - 1);
+      project(ps);
       if (!e.sync_only()) return;
       ps.c0 = ps.c1 = 0;
       ps.a = 1.0;
@@ -715,7 +705,7 @@ struct FlatPass {
     if constexpr (!F64) return e.reduce_all(e.run_pass(ps), fn);
     e.zero_acc();
     if constexpr (AUG) e.aug_begin(ps);
-    project(ps, -1);
+    project(ps);
     return e.reduce_all(e.write_self(ps, 0), fn);
   }
 };

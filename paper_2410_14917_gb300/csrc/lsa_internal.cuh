@@ -142,9 +142,17 @@ __host__ __device__ __forceinline__ long long edge_slot(int tiles_x, int tiles_y
 bool make_devop(const lsa_op* op, DevOp* d);
 Tiling make_tiling(const DevOp& d);
 // Limbs of m basis columns for the flat float64 kernel: columns padded to whole pairs of values, and reads run
-// up to a piece of points past the last one.
+// up to a piece of points past the last one; then the shift bases of their pieces (lsa_fix.cuh), those of a piece's
+// columns in a row, at the row of its first point / 32.
+__host__ __device__ inline size_t limb_values(const DevOp& d, int m) {
+  return (size_t)d.ns * ((d.npts + 1) & ~1LL) * m + 1024;
+}
+__host__ __device__ inline int limb_key_stride(int m) { return (m + 7) & ~7; }
+__device__ inline unsigned* limb_keys(int2* F, const DevOp& d, int m) {
+  return reinterpret_cast<unsigned*>(F + limb_values(d, m));
+}
 inline size_t limb_bytes(const DevOp& d, int m) {
-  return ((size_t)d.ns * ((d.npts + 1) & ~1LL) * m + 1024) * sizeof(int2);
+  return limb_values(d, m) * sizeof(int2) + (size_t)((d.npts + 31) / 32) * limb_key_stride(m) * sizeof(unsigned);
 }
 constexpr size_t kLimbBytes = (size_t)64 << 30;   // larger bases are converted in place
 // Bytes that a call needs at least; lsa_workspace_bytes adds the room for the flat kernel's limbs.  0: bad arguments.

@@ -161,3 +161,43 @@ def test_start_vectors_near_the_ends_of_the_range(path, bits):
 
     ref, y = call(v), call(v * 2.0**bits)
     assert float((y * 2.0**-bits - ref).norm()) <= 1e-14 * float(ref.norm())
+
+
+@pytest.mark.parametrize("path", ["flat", "flat_in_place", "cluster"])
+@pytest.mark.parametrize("background", [1e-2, 1e-4, 1e-7])
+@pytest.mark.parametrize("peaks", [1, 40])
+def test_peaks_over_a_background(path, background, peaks):
+    """The integer sums keep every block's products to half a rounding unit of
+    its vectors' norms (lsa_fix.cuh), so for peaks over a background beta is
+    right to the roundings of some forty float64 additions and a square root
+    (1e-15), and the basis loses orthogonality by rounding alone: as the
+    float64 tile form, within the spread of two orders of its sums (4)."""
+    import paper_2410_14917_gb300 as lsa
+
+    m = 12
+    cfg = W.advdiff2d(64, ny=64, m=m) if path == "cluster" else W.adr3d(128, m=m)
+    op, v = _op(cfg)
+    rng = np.random.default_rng(17)
+    x = background * rng.uniform(-1.0, 1.0, v.numel())
+    x[rng.integers(0, x.size, peaks)] = rng.uniform(0.5, 1.5, peaks)
+    v = torch.from_numpy(x).cuda()
+
+    def run(form):
+        if form == 0 or path == "flat":
+            return _forced(form, lambda: lsa.arnoldi(op, v, m))
+        if path == "cluster":
+            return lsa.arnoldi(op, v, m)
+        w = lsa.Workspace.for_call(op, m, 0)
+        w.nbytes -= 256                  # ends inside the fixed-point basis
+        return _forced(2, lambda: lsa.arnoldi(op, v, m, work=w))
+
+    loss = {}
+    for form in (0, 2):
+        V, H, st = run(form)
+        assert st["m_eff"] == m and st["arnoldi_kernel"] == (0 if form == 0 else 3 if path == "cluster" else 5)
+        V = V[:, :m].T.contiguous()
+        G = V @ V.T - torch.eye(m, dtype=torch.float64, device="cuda")
+        loss[form] = float((G - torch.diag(torch.diag(G))).norm())
+        beta = np.sqrt(np.sum(np.square(x.astype(np.longdouble))))
+        assert abs(st["beta"] / beta - 1) <= 1e-15, form
+    assert loss[2] <= 4.0 * loss[0]
