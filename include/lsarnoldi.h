@@ -488,6 +488,13 @@ lsa_status lsa_read_stats(const void* work, lsa_stats* out, void* stream);
  * <= 10).  Expected result: LSA_ERR_TIMEOUT, with the CUDA context still usable. */
 lsa_status lsa_selftest_barrier_timeout(void* work, size_t work_bytes, double seconds, void* stream);
 
+/* The same for the waits on a counter, each with two CTAs of the three that it
+ * waits for: 1 the barrier of the small exponential, 2 the first wait of a grid
+ * reduction (and of the barrier between two passes), 3 its second wait (grids
+ * of many CTAs).  work: 128 KiB, 256-byte aligned.  Expected result:
+ * LSA_ERR_TIMEOUT; LSA_ERR_NUMERIC when a wait gave up without telling its CTA. */
+lsa_status lsa_selftest_wait_timeout(int wait, void* work, size_t work_bytes, double seconds, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

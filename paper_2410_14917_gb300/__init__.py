@@ -20,7 +20,7 @@ from . import _binding as B
 from ._binding import LsaError, LsaOp, LsaStats, PRECISIONS, VARIANTS, KINDS
 
 __all__ = ["Operator", "phiv", "phiv_lincomb", "phiv_lincomb_adaptive", "axpby", "phiv_noalloc", "arnoldi", "matvec", "expm_phi", "workspace_bytes", "read_stats",
-           "selftest_barrier_timeout", "max_m", "LsaError", "Workspace", "Batch", "phiv_batched",
+           "selftest_barrier_timeout", "selftest_wait_timeout", "max_m", "LsaError", "Workspace", "Batch", "phiv_batched",
            "phiv_vjp", "Phi1GrayScott"]
 
 
@@ -378,6 +378,14 @@ def selftest_barrier_timeout(seconds: float = 0.5, stream=None) -> int:
     work = Workspace(1 << 16)
     return int(B.lib().lsa_selftest_barrier_timeout(ctypes.c_void_p(work.ptr), work.nbytes,
                                                     float(seconds), _stream_ptr(stream)))
+
+
+def selftest_wait_timeout(wait: int, seconds: float = 0.5, stream=None) -> int:
+    """Status of lsa_selftest_wait_timeout: -3 (timeout) when the counter wait
+    1, 2 or 3 gives up after `seconds` as it should."""
+    work = Workspace(1 << 17)
+    return int(B.lib().lsa_selftest_wait_timeout(int(wait), ctypes.c_void_p(work.ptr), work.nbytes,
+                                                 float(seconds), _stream_ptr(stream)))
 
 
 def _op_array(ops):

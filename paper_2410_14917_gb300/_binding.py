@@ -76,6 +76,7 @@ SIGNATURES = {
     "lsa_phiv_noalloc": (c_int, [POINTER(LsaOp), c_void_p, c_double, c_int, c_int, c_double, c_int,
                                  c_int, c_void_p, POINTER(LsaStats), c_void_p]),
     "lsa_selftest_barrier_timeout": (c_int, [c_void_p, c_size_t, c_double, c_void_p]),
+    "lsa_selftest_wait_timeout": (c_int, [c_int, c_void_p, c_size_t, c_double, c_void_p]),
     "lsa_batch_workspace_bytes": (c_size_t, [POINTER(LsaOp), POINTER(c_int), c_int, c_int, c_int]),
     "lsa_batch_create": (c_int, [POINTER(LsaOp), POINTER(c_int), c_int, c_double, c_int, c_double,
                                  c_int, c_int, c_void_p, c_size_t, POINTER(c_void_p), c_void_p]),

@@ -1278,4 +1278,14 @@ lsa_status lsa_selftest_barrier_timeout(void* work, size_t work_bytes, double se
   return fill_stats(ctl, &st, s);
 }
 
+lsa_status lsa_selftest_wait_timeout(int wait, void* work, size_t work_bytes, double seconds, void* stream) {
+  if (wait < 1 || wait > 3 || !(seconds > 0.0) || seconds > 10.0) return LSA_ERR_ARG;
+  if (!work || !aligned256(work) || work_bytes < wait_selftest_bytes()) return LSA_ERR_WORKSPACE;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (launch_wait_selftest(work, wait, (long long)(seconds * 1e9), s) != cudaSuccess) return LSA_ERR_CUDA;
+  lsa_stats st;
+  const lsa_status r = fill_stats(work, &st, s);
+  return r == LSA_ERR_TIMEOUT && st.grid_syncs != 2 ? LSA_ERR_NUMERIC : r;
+}
+
 }  // extern "C"

@@ -188,6 +188,8 @@ cudaError_t launch_init(Ctl* ctl, const DevOp& op, float* g0, float* g1, int pre
 cudaError_t launch_copy_basis(void* Vdst, const void* Vsrc, int precision, long long N, int m,
                               const Ctl* ctl, int apply_sigma, cudaStream_t s);
 cudaError_t launch_timeout_selftest(Ctl* ctl, long long timeout_ns, cudaStream_t s);
+size_t wait_selftest_bytes();
+cudaError_t launch_wait_selftest(void* work, int wait, long long timeout_ns, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Device helpers

@@ -1,8 +1,10 @@
 // Small kernels: workspace initialisation, the augmented Hessenberg exponential
 // (S5), the output combination (S6), basis rescaling for lsa_arnoldi, and the
-// barrier-timeout self-test.
+// wait-timeout self-tests.
 #include <math.h>
+#include <string.h>
 
+#include "lsa_engine.cuh"
 #include "lsa_expm.cuh"
 
 namespace lsa {
@@ -155,6 +157,47 @@ __global__ void k_timeout_selftest(Ctl* ctl, long long timeout_ns) {
 
 cudaError_t launch_timeout_selftest(Ctl* ctl, long long timeout_ns, cudaStream_t s) {
   k_timeout_selftest<<<2, 32, 0, s>>>(ctl, timeout_ns);
+  return cudaGetLastError();
+}
+
+// The waits on a counter, with two CTAs and a target that one more CTA would
+// have to reach: 1 the small exponential's group barrier, 2 the first wait of
+// Engine::reduce_all (also that of the barrier between two passes and of the
+// placement), 3 its second wait, for the sums of a grid of many rows.  Counts
+// the CTAs whose wait returned false.
+__global__ void __launch_bounds__(NT) k_wait_selftest(ArnoldiParams P, int wait) {
+  using E = Engine<OpAdvDiff2D, double, double, false, false>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  bool ok;
+  if (wait == 1) {
+    __shared__ int flag;
+    ok = counter_barrier(expm_barrier(P.ctl), gridDim.x + 1u, &flag, P.timeout_ns);
+  } else {
+    E e(P, *reinterpret_cast<E::Smem*>(smem_raw), reinterpret_cast<double*>(smem_raw + E::small_offset()));
+    e.redundant_steps();
+    if (wait == 2) e.gsize = (int)gridDim.x + 1;
+    else e.nrows = E::DIRECT + 1;               // 3: the two CTAs sum 8 of 12 slots
+    ok = e.reduce_all(12, [] {});
+  }
+  if (!ok && threadIdx.x == 0) atomicAdd(&P.ctl->syncs, 1);
+}
+
+size_t wait_selftest_bytes() {
+  return sizeof(Ctl) + 256 + (size_t)(Engine<OpAdvDiff2D, double, double, false, false>::DIRECT + 2) * SLOTS * sizeof(double);
+}
+cudaError_t launch_wait_selftest(void* work, int wait, long long timeout_ns, cudaStream_t s) {
+  using E = Engine<OpAdvDiff2D, double, double, false, false>;
+  ArnoldiParams P;
+  memset(&P, 0, sizeof(P));
+  P.ctl = (Ctl*)work;
+  P.partials = (double*)((char*)work + ((sizeof(Ctl) + 255) & ~(size_t)255));
+  P.gsum = P.partials + (size_t)(E::DIRECT + 1) * SLOTS;
+  P.timeout_ns = timeout_ns;
+  const size_t sm = E::smem_bytes();
+  cudaError_t e = cudaFuncSetAttribute(k_wait_selftest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e == cudaSuccess) e = cudaMemsetAsync(work, 0, wait_selftest_bytes(), s);
+  if (e != cudaSuccess) return e;
+  k_wait_selftest<<<2, NT, sm, s>>>(P, wait);
   return cudaGetLastError();
 }
 

@@ -133,6 +133,25 @@ def test_barrier_timeout_returns_error_and_context_survives():
     assert max(rel_errors(y, ref)) < FP64_TOL
 
 
+@pytest.mark.parametrize("wait", [1, 2, 3])
+def test_counter_waits_give_up_and_context_survives(wait):
+    """The small exponential's barrier and both waits of the grid reduction,
+    each short of one arrival: they end after the limit, record the timeout
+    and return false in every CTA."""
+    import time
+
+    import paper_2410_14917_gb300 as lsa
+
+    lsa.selftest_wait_timeout(wait, 0.01)                  # (loads the kernel)
+    t0 = time.perf_counter()
+    assert lsa.selftest_wait_timeout(wait, 0.2) == -3      # LSA_ERR_TIMEOUT
+    assert 0.2 <= time.perf_counter() - t0 < 2.0
+    cfg = W.advdiff2d(16, m=8, p=1)
+    y, st, inp = run(cfg, "hcwy", "fp64")
+    ref, _ = oracle_phiv(cfg)
+    assert max(rel_errors(y, ref)) < FP64_TOL
+
+
 def test_norm_estimate_fallback_path():
     """Diagonal operators (3D ADR with no diffusion or advection) with three
     eigenvalue clusters of width delta: the Krylov space is nearly exhausted
