@@ -419,7 +419,7 @@ lsa_status lsa_phiv_vjp(const lsa_op* op, const double* v, double h, int m, int 
  * cost.  group_size = lsa_batch_info's ctas with nlarge = count is one grid
  * per instance; nlarge = 0 is one CTA per instance.  lsa_batch_tune times a
  * set of tilings on the caller's data and keeps the fastest, then (hybrid
- * variants) the other step form on that tiling, and keeps the faster. */
+ * variants) the other step forms on that tiling, and keeps the fastest. */
 typedef struct lsa_batch lsa_batch;
 
 /* Device workspace bytes for a batch (0 if the arguments are invalid).
@@ -442,13 +442,19 @@ lsa_status lsa_batch_info(const lsa_batch* plan, int* ctas, int* group_size, int
 /* Set the tiling: 1 <= group_size <= ctas, 0 <= nlarge <= count. */
 lsa_status lsa_batch_set_tiling(lsa_batch* plan, int group_size, int nlarge);
 
-/* Step form of the hybrid variants in this plan (see lsa_tune_step): 0 the
- * one-pass step, 1 the two-phase step (the default for the hybrid variants;
- * its extra barrier is counted over an instance's group).  Both compute
- * bitwise the same result.
- * lsa_batch_step_form returns the plan's form (-1 for a null plan). */
-lsa_status lsa_batch_set_step_form(lsa_batch* plan, int two_phase);
+/* Step form of the hybrid variants in this plan (see lsa_tune_step; a barrier
+ * between passes is counted over an instance's group): 0 the one-pass step, 1
+ * the two-phase step over tiles, 2 the flat two-phase step (float64 plans of the
+ * hybrid variants; LSA_ERR_ARG for others).  Forms 0 and 1 compute bitwise the
+ * same result, form 2 the same to rounding.  New plans of the hybrid variants
+ * run form 2 in float64 and form 1 with the float32 basis.
+ * lsa_batch_step_form returns 0 for the one-pass step and 1 for either two-phase
+ * form (-1 for a null plan), and setting form 1 leaves a plan that runs form 2
+ * as it is, so that what was read can be set again; to reach the tile passes
+ * from form 2 set 0, then 1.  lsa_batch_step_passes returns the form itself. */
+lsa_status lsa_batch_set_step_form(lsa_batch* plan, int form);
 int lsa_batch_step_form(const lsa_batch* plan);
+int lsa_batch_step_passes(const lsa_batch* plan);
 
 /* Enqueue one batched evaluation on `stream` (two kernels: initialisation and
  * the persistent kernel; nothing is read back).  use_graph != 0 captures the
@@ -466,7 +472,7 @@ lsa_status lsa_batch_read_stats(const lsa_batch* plan, lsa_stats* stats, int* fi
 /* Time candidate tilings (one CTA per instance, one grid per instance, and
  * groups of 2..32 CTAs for the costliest count/64 .. count instances), each
  * `reps` times after one warm-up run on the caller's v and y, keep the fastest
- * and return it (with, for the hybrid variants, the faster step form on it,
+ * and return it (with, for the hybrid variants, the fastest step form on it,
  * see lsa_batch_step_form).  Synchronises `stream`; overwrites y. */
 lsa_status lsa_batch_tune(lsa_batch* plan, const double* v, double* y, int reps, int* group_size,
                           int* nlarge, float* ms_best, void* stream);

@@ -442,10 +442,16 @@ class Batch:
 
     @property
     def step_form(self):
-        """1 when the plan runs the two-phase hybrid step, 0 for the one-pass step."""
+        """1 when the plan runs a two-phase hybrid step, 0 for the one-pass step."""
         return int(B.lib().lsa_batch_step_form(self._h))
 
+    @property
+    def step_passes(self):
+        """The form itself: 0 one-pass, 1 two-phase over tiles, 2 flat two-phase."""
+        return int(B.lib().lsa_batch_step_passes(self._h))
+
     def set_step_form(self, two_phase: int):
+        """0, 1 or 2 (float64 plans of the hybrid variants); 1 leaves a plan that runs form 2 as it is."""
         _check(B.lib().lsa_batch_set_step_form(self._h, int(two_phase)), "lsa_batch_set_step_form",
                ok=(B.LSA_OK,))
 

@@ -339,13 +339,17 @@ lsa_status lsa_batch_set_tiling(lsa_batch* b, int group_size, int nlarge) {
   return LSA_OK;
 }
 
-lsa_status lsa_batch_set_step_form(lsa_batch* b, int two_phase) {
-  if (!b || (two_phase != 0 && two_phase != 1)) return LSA_ERR_ARG;
-  b->step = two_phase;
+lsa_status lsa_batch_set_step_form(lsa_batch* b, int form) {
+  if (!b || form < 0 || form > 2) return LSA_ERR_ARG;
+  if (form == 2 && (b->precision != LSA_FP64 || !is_hybrid(b->variant))) return LSA_ERR_ARG;
+  if (form == 1 && b->step == 2) return LSA_OK;      // (a two-phase form already: what lsa_batch_step_form reads)
+  b->step = form;
   return LSA_OK;
 }
 
 int lsa_batch_step_form(const lsa_batch* b) { return b ? (b->step ? 1 : 0) : -1; }
+
+int lsa_batch_step_passes(const lsa_batch* b) { return b ? b->step : -1; }
 
 lsa_status lsa_batch_run(lsa_batch* b, const double* v, double* y, int use_graph, void* stream) {
   if (!b || !v || !y) return LSA_ERR_ARG;

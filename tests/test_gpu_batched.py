@@ -251,3 +251,32 @@ def test_batched_default_step_form(variant):
     torch.cuda.synchronize()
     _check_instances(b, y, SMALL, variant, FP64_TOL)
     b.close()
+
+
+@pytest.mark.parametrize("precision,variant,forms", [("fp64", "hcwy", (0, 1, 2)), ("fp32", "hcwy", (0, 1)),
+                                                     ("fp64", "mgs", (0, 1))])
+def test_step_form_names_what_runs(precision, variant, forms):
+    """step_passes tells the tile and the flat two-phase forms apart, setting
+    what step_form reads changes nothing, and every form of a plan can be
+    reached again."""
+    lsa = _lsa()
+    b, v, _ = _batch(SMALL, variant, precision)
+    default = {"fp64": 2, "fp32": 1}[precision] if variant == "hcwy" else 0
+    assert b.step_passes == default
+    y = b.run(v, graph=False).clone()
+    b.set_step_form(b.step_form)
+    assert b.step_passes == default
+    torch.cuda.synchronize()
+    assert torch.equal(b.run(v, graph=False), y)
+    for f in range(3):
+        if f not in forms:
+            with pytest.raises(lsa.LsaError):
+                b.set_step_form(f)
+            continue
+        b.set_step_form(f)
+        assert b.step_passes == f and b.step_form == min(f, 1)
+    b.set_step_form(default)
+    if default != 1:
+        assert b.step_passes == default
+        assert torch.equal(b.run(v, graph=False), y)
+    b.close()
