@@ -60,3 +60,17 @@ def test_fp32_roofline_object(kind, kernel):
     assert r["kernel"].startswith(kernel + " ")
     assert r["achieved"] == pytest.approx(r["algorithmic_bytes"] / 29.0e-3 / 1e9)
     assert r["frac"] == pytest.approx(r["achieved"] / hbm)
+
+
+def test_integer_sums_count_the_float64_unit_alone():
+    """Where the inner products are integer sums the fraction is the float64
+    unit's: the FMAs of the projection, the stencil and w . w over its peak."""
+    cfg = W.config(1)
+    N, m, taps = W.n_dof(cfg), 64, 7
+    unit = bench.float64_unit_flops(cfg, m)
+    assert unit == (m * (m - 1) + m * (2 + 2 * taps) + 2 * m + 2) * N
+    _, flops = bench.algorithmic_counts(cfg, "fp64", m)
+    pk, src = bench.integer_sums_peak(1.05, "test peak", flops, unit)
+    r = bench.phiv_roofline(cfg, "fp64", "hcwy", 5.7, m, 5, pk, src)
+    assert r["frac"] == pytest.approx(unit / 5.7e-3 / 1e12 / 1.05) and r["frac"] < 1.0
+    assert bench.adjoint_flops(cfg, m, unit) == 8 * unit
