@@ -143,6 +143,10 @@ long long lsa_op_dof(const lsa_op* op);
  * take a workspace without that part and then convert the columns at each use. */
 size_t lsa_workspace_bytes(const lsa_op* op, int m, int p, int precision);
 
+/* The size without that part: the least that those calls take (the same as
+ * lsa_workspace_bytes with the float32 basis and for bases beyond 64 GiB). */
+size_t lsa_workspace_least_bytes(const lsa_op* op, int m, int p, int precision);
+
 /* S1 alone: y = A x.  x, y: dev, N elements of the basis type (double for
  * LSA_FP64, float for LSA_FP32_BASIS).  Uses the same stencil code as the
  * Arnoldi kernels.  work: dev workspace of lsa_workspace_bytes(op, 1, 0, precision). */

@@ -97,8 +97,11 @@ def max_m() -> int:
     return int(B.lib().lsa_max_m())
 
 
-def workspace_bytes(op: Operator, m: int, p: int = 0, precision: str = "fp64") -> int:
-    n = B.lib().lsa_workspace_bytes(ctypes.byref(op.c), int(m), int(p), PRECISIONS[precision])
+def workspace_bytes(op: Operator, m: int, p: int = 0, precision: str = "fp64", least: bool = False) -> int:
+    """Bytes of a call's workspace; least: without the room for the fixed-point
+    copy of a float64 basis, which a call can do without at some cost in time."""
+    f = B.lib().lsa_workspace_least_bytes if least else B.lib().lsa_workspace_bytes
+    n = f(ctypes.byref(op.c), int(m), int(p), PRECISIONS[precision])
     if n == 0:
         raise LsaError(B.LSA_ERR_ARG, "lsa_workspace_bytes")
     return int(n)
@@ -115,7 +118,11 @@ class Workspace:
 
     @classmethod
     def for_call(cls, op, m, p=0, precision="fp64"):
-        return cls(workspace_bytes(op, m, p, precision))
+        """The full workspace of a call, or the least one when the device has no room for it."""
+        try:
+            return cls(workspace_bytes(op, m, p, precision))
+        except torch.OutOfMemoryError:
+            return cls(workspace_bytes(op, m, p, precision, least=True))
 
 
 def _check(st, what, ok=(B.LSA_OK, B.LSA_BREAKDOWN, B.LSA_NOT_CONVERGED)):

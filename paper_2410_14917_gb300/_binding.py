@@ -45,6 +45,7 @@ SIGNATURES = {
     "lsa_version": (c_int, []),
     "lsa_status_string": (c_char_p, [c_int]),
     "lsa_op_dof": (c_longlong, [POINTER(LsaOp)]),
+    "lsa_workspace_least_bytes": (c_size_t, [POINTER(LsaOp), c_int, c_int, c_int]),
     "lsa_workspace_bytes": (c_size_t, [POINTER(LsaOp), c_int, c_int, c_int]),
     "lsa_matvec": (c_int, [POINTER(LsaOp), c_void_p, c_void_p, c_int, c_void_p, c_size_t, c_void_p]),
     "lsa_arnoldi": (c_int, [POINTER(LsaOp), c_void_p, c_int, c_int, c_int, c_void_p, c_void_p,

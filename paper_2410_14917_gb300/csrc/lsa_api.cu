@@ -573,11 +573,6 @@ static bool workspace_layout(const lsa_op* op, int m, int p, int precision, Layo
   return make_layout(d, m, precision, L);
 }
 
-size_t workspace_least_bytes(const lsa_op* op, int m, int p, int precision) {
-  Layout L;
-  return workspace_layout(op, m, p, precision, &L) ? L.base : 0;
-}
-
 }  // namespace lsa
 
 using namespace lsa;
@@ -610,6 +605,11 @@ long long lsa_op_dof(const lsa_op* op) {
 size_t lsa_workspace_bytes(const lsa_op* op, int m, int p, int precision) {
   Layout L;
   return workspace_layout(op, m, p, precision, &L) ? L.total : 0;
+}
+
+size_t lsa_workspace_least_bytes(const lsa_op* op, int m, int p, int precision) {
+  Layout L;
+  return workspace_layout(op, m, p, precision, &L) ? L.base : 0;
 }
 
 lsa_status lsa_matvec(const lsa_op* op, const void* x, void* y, int precision, void* work,

@@ -155,8 +155,6 @@ inline size_t limb_bytes(const DevOp& d, int m) {
   return limb_values(d, m) * sizeof(int2) + (size_t)((d.npts + 31) / 32) * limb_key_stride(m) * sizeof(unsigned);
 }
 constexpr size_t kLimbBytes = (size_t)64 << 30;   // larger bases are converted in place
-// Bytes that a call needs at least; lsa_workspace_bytes adds the room for the flat kernel's limbs.  0: bad arguments.
-size_t workspace_least_bytes(const lsa_op* op, int m, int p, int precision);
 
 // Launchers implemented per operator translation unit.
 cudaError_t launch_arnoldi(const ArnoldiParams& P, int precision, int G, cudaStream_t s);

@@ -50,7 +50,7 @@ extern "C" lsa_status lsa_phiv_noalloc(const lsa_op* op, const double* v, double
   const long long N = lsa_op_dof(op);
   if (N < 1 || m < 1) return LSA_ERR_ARG;
   const int m_used = (m > N) ? (int)N : m;
-  const size_t need = lsa::workspace_least_bytes(op, m_used, p, precision);
+  const size_t need = lsa_workspace_least_bytes(op, m_used, p, precision);
   if (need == 0) return LSA_ERR_ARG;
   if (need > kStaticBytes) return LSA_ERR_WORKSPACE;   // beyond the fixed maximum
   lsa_status st = lsa_phiv(op, v, h, p, m, tol, variant, precision, y, work, kStaticBytes,

@@ -201,3 +201,32 @@ def test_peaks_over_a_background(path, background, peaks):
         beta = np.sqrt(np.sum(np.square(x.astype(np.longdouble))))
         assert abs(st["beta"] / beta - 1) <= 1e-15, form
     assert loss[2] <= 4.0 * loss[0]
+
+
+def test_least_workspace(monkeypatch):
+    """lsa_workspace_least_bytes leaves out the fixed-point basis alone: calls
+    take that much and no less, and Workspace.for_call falls back to it when
+    the device has no room for the full one."""
+    import paper_2410_14917_gb300 as lsa
+
+    op, v = _op(W.advdiff2d(201, ny=203, m=20, p=1))
+    full, least = (lsa.workspace_bytes(op, 20, 1, least=x) for x in (False, True))
+    assert 8 * 20 * op.N <= full - least <= 8 * 20 * op.N * 1.05 + 65536
+    assert lsa.workspace_bytes(op, 20, 1, "fp32", least=True) == lsa.workspace_bytes(op, 20, 1, "fp32")
+    ref, _ = _forced(2, lambda: lsa.phiv(op, v, 1e-2, 1, 20))
+    empty = torch.empty
+
+    def short(n, *args, **kw):
+        if kw.get("dtype") == torch.uint8 and n >= full:
+            raise torch.OutOfMemoryError("no room")
+        return empty(n, *args, **kw)
+
+    monkeypatch.setattr(torch, "empty", short)
+    w = lsa.Workspace.for_call(op, 20, 1)
+    monkeypatch.undo()
+    assert w.nbytes == least
+    y, _ = _forced(2, lambda: lsa.phiv(op, v, 1e-2, 1, 20, work=w))
+    assert float((y - ref).norm()) <= 1e-12 * float(ref.norm())
+    w.nbytes -= 256
+    with pytest.raises(lsa.LsaError):
+        lsa.phiv(op, v, 1e-2, 1, 20, work=w)
