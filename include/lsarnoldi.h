@@ -107,7 +107,9 @@ typedef struct {
   int breakdown;          /* 1 after a lucky breakdown */
   int norm_fallbacks;     /* explicit-norm fallbacks of the hybrid norm estimate (Alg. 4) */
   int grid_syncs;         /* global reductions performed (in-kernel grid barriers with reduction) */
-  int grid_barriers;      /* all grid barriers, including those without a reduction */
+  int grid_barriers;      /* the reductions and, with a two-phase step, the barriers between a step's projection
+                             and its second pass (a reduction counts once however many waits it takes; the
+                             float32 flat passes' barrier after the stencil is not counted) */
   double beta;            /* ||v|| */
   double err_est;         /* beta*h*H_{m+1,m}*|e_m^T phi_{p+1}(h H_m) e_1| (phiv only) */
   double h_last;          /* H_{m+1,m} */
@@ -189,8 +191,8 @@ lsa_status lsa_arnoldi(const lsa_op* op, const double* v, int m, int variant, in
  * operator kind and grid, m, variant and precision use it (process-wide
  * table, thread-safe).  LSA_TWO_PHASE=0, 1 or 2 in the environment overrides
  * the table (2 runs form 1 where form 2 does not apply).  Without either:
- * form 2 for float64 3D grids and for 2D grids of at least six 16 x 16 tiles
- * per SM, form 1 for float32-basis 3D grids, form 0 otherwise (the
+ * form 2 in float64; with the float32 basis form 2 for 2D grids of at least six
+ * 16 x 16 tiles per SM, form 1 for 3D grids and form 0 otherwise (the
  * crossovers measured on GB300).
  *  v      dev, N doubles: start vector of the timing runs (not modified).
  *  work   dev workspace of lsa_workspace_bytes(op, m, 0, precision).

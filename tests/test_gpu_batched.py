@@ -280,3 +280,32 @@ def test_step_form_names_what_runs(precision, variant, forms):
         assert b.step_passes == default
         assert torch.equal(b.run(v, graph=False), y)
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("kind", ["grayscott2d", "adr3d"])
+def test_other_operators_equal_single_calls(kind, precision):
+    """Batches of the two-species and the 3D operator: every instance against
+    the single call, with one CTA, groups and the whole grid per instance."""
+    lsa = _lsa()
+    g = torch.Generator(device="cuda").manual_seed(23)
+    rand = lambda n: torch.rand(n, dtype=torch.float64, device="cuda", generator=g)
+    ops, ms = [], [12, 30, 17, 24, 9]
+    for nx, ny, nz in [(5, 7, 3), (48, 33, 5), (32, 32, 8), (17, 64, 16), (70, 41, 4)]:
+        if kind == "grayscott2d":
+            ops.append(lsa.Operator.grayscott2d(nx * nz, ny, 2.5 / (nx * nz), 2e-5, 1e-5, 0.04, 0.06, rand(nx * ny * nz),
+                                                rand(nx * ny * nz)))
+        else:
+            ops.append(lsa.Operator.adr3d(nx, ny, nz, 1.0 / nx, 1e-3, (1.0, 1.0, 1.0), -rand(nx * ny * nz)))
+    vs = [rand(op.N) - 0.5 for op in ops]
+    tol = 1e-12 if precision == "fp64" else 1e-5
+    b = lsa.Batch(ops, ms, 5e-3, 1, precision=precision)
+    refs = [lsa.phiv(op, v, 5e-3, 1, m, precision=precision)[0] for op, v, m in zip(ops, vs, ms)]
+    for gs, nl in [(1, 0), (4, 3), (b.ctas, b.count)]:
+        b.set_tiling(gs, nl)
+        y = b.run(torch.cat(vs), graph=False)
+        st, fin, _ = b.stats()
+        assert st >= 0 and fin == b.count
+        for part, ref in zip(b.split(y), refs):
+            assert float((part - ref).norm()) <= tol * float(ref.norm())
+    b.close()
