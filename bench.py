@@ -54,7 +54,7 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # ((256/192)^3) (profiles/k_arnoldi_stream_adr3d_192_fp32.md).
 PROFILED_TRAFFIC = {("grayscott2d_512", "fp64", "hcwy", 0): 9.118409e9 + 0.744297e9,
                     ("grayscott2d_512", "fp64", "hcwy", 4): 13.717263e9 + 0.777655e9,
-                    ("grayscott2d_512", "fp64", "hcwy", 5): 17.076877e9 + 0.787758e9,
+                    ("grayscott2d_512", "fp64", "hcwy", 5): 17.129904e9 + 0.789721e9,
                     ("adr3d_256", "fp32", "hcwy", 2): (28.712327e9 + 2.551436e9) * (256 / 192) ** 3}
 
 

@@ -300,7 +300,7 @@ static int flat_ctas_per_sm(const ArnoldiParams& P, int precision) {
 
 // Where nothing is recorded or forced, the flat kernel runs
 //  * in float64 at every size (a phi product on GB300, flat against one-pass:
-//    Gray-Scott 48^2 0.61 and 0.80 ms, 256^2 1.7 and 2.1, 512^2 5.6 and 9.6;
+//    Gray-Scott 48^2 0.61 and 0.80 ms, 256^2 1.7 and 2.1, 512^2 5.7 and 9.6;
 //    advection-diffusion 97 x 61 0.41 and 0.46; ADR 16^3 0.36 and 0.82);
 //  * with the float32 basis on 2D grids of at least six 16 x 16 tiles per SM
 //    (Gray-Scott 512^2 2.1 against 4.4 ms; below that, and on 3D grids that the

@@ -2,7 +2,7 @@
 // layout, cost order), the CTA-group tiling and its tuner, CUDA-graph capture
 // and replay, and the per-instance statistics.  The device code is in
 // lsa_batched.cuh; the kernels are instantiated per operator in
-// lsa_arnoldi_<op>.cu.
+// lsa_batched_<op>.cu.
 #include <math.h>
 #include <string.h>
 

@@ -8,14 +8,16 @@
 // forms of the hybrid step, projected once over flat shares and read back
 // after a grid barrier, by the tiles or, in the flat form, over flat shares
 // of the points again), and accumulates inner products of basis columns with
-// x and/or w.  The per-CTA partial sums go to
-// global memory, and one grid barrier reduces them in two levels: the last CTA
-// of each group of RG CTAs sums its group, the last group sums the group rows
-// (both in a fixed order: deterministic) and does the small O(j^2)
+// x and/or w.  The per-CTA partial sums go to global memory; after one grid
+// barrier every CTA sums them (up to DIRECT rows), or after it CTA q sums four
+// slots of all rows and a second barrier lets every CTA read the sums (both in a
+// fixed order: deterministic).  Then every CTA does the small O(j^2)
 // double-precision work of the step (H column, correction matrix T, norm
-// estimate) before releasing the others.  (The batched form, whose groups are
-// instances, sums all its CTAs' partials in one level.)  A global reduction of the paper
-// (an MPI_Allreduce, Sect. 2.3) is therefore one grid barrier here.
+// estimate) on the same numbers, and the lead one writes the results, so that
+// nothing is published after it.  (The TMA-staged and streaming kernels reduce in
+// two levels instead, groups of RG CTAs and their sums, and the last CTA takes the
+// step and releases the others: reduce_step.)  A global reduction of the paper (an
+// MPI_Allreduce, Sect. 2.3) is one or two grid barriers here.
 #pragma once
 
 #include "lsa_ops.cuh"

@@ -18,7 +18,7 @@
 // stencil (float64 unit) from another's inner products (integer unit, memory:
 // lsa_fix.cuh).  The columns come through a ring of asynchronous copies, in
 // which a warp keeps 6 KB in flight (in registers, 2 to 4 KB: ADR 256^3 70 against
-// 73 ms a phi product; with the limbs kept instead of converted 56 ms; the float64
+// 73 ms a phi product; with the limbs kept instead of converted 55 ms; the float64
 // products it replaces took 94).  It walks its share backwards, so that it
 // starts on the x that pass A left in L2 (and, where the columns are converted in
 // place, on theirs).

@@ -25,8 +25,9 @@ constexpr int RG = 32;                    // CTAs per group of the two-level gri
 constexpr int RG_MAX = 64;                // groups of the two-level grid reduction (G <= RG * RG_MAX)
 constexpr int SMID_CAP = 256;             // SM ids tracked by the SM-aware placement
 
-// Device-side control block, one per workspace.  Written only by the CTA that
-// arrives last at a grid barrier (between barriers), read by all after it.
+// Device-side control block, one per workspace.  Written by the lead CTA of the
+// grid kernels, where every CTA takes the step, and by the CTA that arrives last at
+// a barrier of the TMA-staged and streaming kernels, read by all after it.
 struct Ctl {
   unsigned int arrive;     // grid-barrier arrivals (monotonic within a launch)
   unsigned int release;    // last released barrier generation
